@@ -68,7 +68,6 @@ TRAFFIC_PER_LAUNCH = {
     # curved LV-like slab at full size: the eight ticks of one barrier step
     ("lv3d", "k_tick_mapped<float,3,1>"): 4.4873e7,
     # 3D slab: the quarter slab's eight ticks, tick 0 and tick 4 scaled to the full slab
-    ("slab3d", "k_tick_tc<3,2>"): 1.9601e9,
 }
 # Mapped Q1 3D (lv3d): per element step the state 128 B, metadata and the RV-T accumulator
 # 49 B, and the element's geometric factors (8 nodes x 7 values + 6 faces x 4 points x 5
@@ -214,8 +213,10 @@ def run_ours(args, rank, world):
         kname = "k_tick_mapped" + kname
     elif args.sweep == "group" and prob_order(factory) == 1:
         kname = "k_tick_group" + kname.replace(",1>", ">")
-    elif args.sweep == "tensor" or (args.sweep == "default" and factory().order == 2 and factory().dim == 3):
+    elif args.sweep == "tensor":
         kname = "k_tick_tc<3,2>"
+    elif args.sweep in ("default", "thread") and factory().order == 2 and factory().dim == 3:
+        kname = "k_tick_q23<3,2>"
     else:
         kname = ("k_sweep" if args.sweep == "coop" else "k_tick") + kname
     prob = factory()
@@ -307,7 +308,7 @@ def run_ours(args, rank, world):
             "warmup": args.warmup, "ms_per_step": total_ms_all / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {"workload": workload_name(prob),
-                       "sweep": args.sweep if args.sweep != "default" else ("tensor" if "k_tick_tc" in kname else "thread"),
+                       "sweep": args.sweep if args.sweep != "default" else "thread",
                        "tick_shape": args.tick_shape or "128,16",
                        "domain_cm": list(prob.extent[:prob.dim]), "base": list(prob.base[:prob.dim]),
                        "max_refine": prob.max_refine, "n_lts_levels": prob.n_lts_levels,
@@ -860,7 +861,7 @@ def main():
     ap.add_argument("--tick-shape", default="", help="sweep launch shape 'threads,blocks_per_sm'")
     ap.add_argument("--base", default="", help="base grid 'nx,ny[,nz]' at the workload's element size")
     ap.add_argument("--sweep", default="default", choices=["default"] + sorted(SWEEPS),
-                    help="sweep kernel variant (default: the library's choice, tensor for Q2 3D FP32 and "
+                    help="sweep kernel variant (default: the library's choice, thread; "
                          "thread otherwise; thread per element; group: Q1 lanes per element; coop: one "
                          "cooperative launch per barrier; tensor: tcgen05 residual, Q2 3D FP32)")
     args = ap.parse_args()

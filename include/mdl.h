@@ -240,14 +240,13 @@ int mdl_set_tick_shape(mdl_ctx* ctx, int32_t threads, int32_t blocks_per_sm);
 /* Sweep kernel variant.  All follow Alg. 1 tick by tick; THREAD and COOP run the same
  * per-element arithmetic, GROUP sums the face terms in another order; they agree to the
  * working precision's rounding:
- *   MDL_SWEEP_THREAD  one thread per due element, one launch per tick; the default except
- *                     for Q2 3D FP32 contexts, whose default is MDL_SWEEP_TENSOR;
+ *   MDL_SWEEP_THREAD  one thread per due element, one launch per tick; the default;
  *   MDL_SWEEP_GROUP   Q1 only: (p+1)^d lanes per element, one lane per face and per DOF,
  *                     one launch per tick (Q2 contexts use MDL_SWEEP_THREAD);
  *   MDL_SWEEP_COOP    every tick and the barrier epilogue in one cooperative launch with
  *                     grid-wide barriers between ticks (bounded waits: one that gives up
  *                     makes the stepping call return MDL_E_TIMEOUT);
- *   MDL_SWEEP_TENSOR  Q2 3D FP32 contexts only (their default): per tile of 64 due
+ *   MDL_SWEEP_TENSOR  Q2 3D FP32 contexts only: per tile of 64 due
  *                     elements the SIPG residual of elements with same-level neighbours is
  *                     one tcgen05 tensor-core product of the gathered element and face-
  *                     neighbour values with the level-0 operator (Sec. 2.1: box elements, so

@@ -36,6 +36,7 @@
 #include "mdl_geometry.h"
 #include "mdl_mapped.cuh"
 #include "mdl_mesh.h"
+#include "mdl_q23.cuh"
 #include "mdl_tables.h"
 #include "mdl_tc.cuh"
 
@@ -112,6 +113,7 @@ class Ctx : public CtxBase {
     Phys<double> phd{};
     Tables<R> T{};
     Phys<R> ph{};
+    OpT<R, DIM, P> op{};
     Grid grid_{};
     StimBoxes sboxes{};
     StimArgs stim{};
@@ -151,6 +153,7 @@ class Ctx : public CtxBase {
     DBuf<DevMeta> meta;
     DBuf<Tables<R>> dT;       // device copies of the tables and physics (fused batch sweeps)
     DBuf<Phys<R>> dph;
+    DBuf<OpT<R, DIM, P>> dop;
     int fused_cur = 0;        // state set the fused sweep of the barrier in flight updates
     bool fused_own = false;   // this round's sweep is the context's own (fused_own_sweep)
     DevMeta* hmeta = nullptr;
@@ -511,7 +514,7 @@ class Ctx : public CtxBase {
                 cfg.attrs = attr;
                 cfg.numAttrs = 1;
                 MDL_CK(cudaMemsetAsync((char*)meta.p + offsetof(DevMeta, gbar), 0, sizeof(unsigned int), st));
-                MDL_CK(cudaLaunchKernelEx(&cfg, k_sweep<R, DIM, P>, ta, T, ph, (const double*)mtab.p));
+                MDL_CK(cudaLaunchKernelEx(&cfg, k_sweep<R, DIM, P>, ta, T, ph, op, (const double*)mtab.p));
                 MDL_LAUNCHED();
                 stats.tick_launches += nt;
                 return MDL_OK;
@@ -546,13 +549,27 @@ class Ctx : public CtxBase {
                     return MDL_OK;
                 }
             }
+            if constexpr (tensor_capable) {
+                // resident blocks only: each walks its due elements, fetching metadata a step ahead
+                const int smem = q23::smem_bytes(tick_threads);
+                int occ = 0;
+                MDL_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tick_q23<DIM, P>, tick_threads, smem));
+                const int gq = std::min(gt, nsm * std::max(1, occ));
+                for (int i = 0; i < nt; ++i) {
+                    ta.tick = i;
+                    MDL_CK(launch_kxs(pdl && i > 0, (size_t)smem, (k_tick_q23<DIM, P>), gq, tick_threads, ta, T, ph, op));
+                    MDL_LAUNCHED();
+                    stats.tick_launches++;
+                }
+                return MDL_OK;
+            }
             for (int i = 0; i < nt; ++i) {
                 ta.tick = i;
                 if constexpr (P == 1) {
                     if (group_tick) MDL_CK(launch_k((k_tick_group<R, DIM>), gt, tick_threads, ta, ph, T));
-                    else MDL_CK(launch_kx(pdl && i > 0, (k_tick<R, DIM, P>), gt, tick_threads, ta, T, ph));
+                    else MDL_CK(launch_kx(pdl && i > 0, (k_tick<R, DIM, P>), gt, tick_threads, ta, T, ph, op));
                 } else {
-                    MDL_CK(launch_kx(pdl && i > 0, (k_tick<R, DIM, P>), gt, tick_threads, ta, T, ph));
+                    MDL_CK(launch_kx(pdl && i > 0, (k_tick<R, DIM, P>), gt, tick_threads, ta, T, ph, op));
                 }
                 MDL_LAUNCHED();
                 stats.tick_launches++;
@@ -672,7 +689,7 @@ public:
         bcfl.release(); info.release(); loc.release(); nbr.release(); hang.release(); root.release();
         order.release();
         for (auto& m : smask) m.release();
-        lvl_ovr.release(); eta_t_ovr.release(); meta.release(); mtab.release(); dT.release(); dph.release();
+        lvl_ovr.release(); eta_t_ovr.release(); meta.release(); mtab.release(); dT.release(); dph.release(); dop.release();
         qvol.release(); qface.release(); qkelly.release(); tcB.release(); tcC.release();
         if (hmeta) cudaFreeHost(hmeta);
         for (auto e : evpool) cudaEventDestroy(e);
@@ -682,13 +699,16 @@ public:
     int create(const mdl_problem& p) override {
         pb = p;
         mapped = pb.geometry != MDL_GEOMETRY_BOX;
-        // Q2 3D FP32: the tensor-core sweep is the default (box elements)
-        tensor_tick = tensor_capable && !mapped;
         B = pb.lts_enabled ? pb.n_lts_levels - 1 : 0;
         make_tables(P, &Td);
         make_phys(pb, Td, &phd);
         convert_tables<R>(Td, &T);
         convert_phys<R>(phd, &ph);
+        if constexpr (P != 1) {
+            BoxOp<double> opd;
+            make_boxop(Td, phd, DIM, P, &opd);
+            convert_boxop<R>(opd, &op);
+        }
         MappedFactors mf;
         if (mapped) {
             const int rc = mapped_factors(pb, Td, &mf, &err);
@@ -767,10 +787,19 @@ public:
                 for (int k = 0; k < DIM; ++k) w *= Td.w[digit<N1>(q, k)];
                 hm[l * NP + q] = w;
             }
-        if (P == 1) {
+        if constexpr (P == 1) {
             std::vector<double> bv, bf, bk;
             q1_blocks(Td, phd, DIM, pb.max_refine, &bv, &bf, &bk);
             std::vector<R> rv(bv.begin(), bv.end()), rf(bf.begin(), bf.end()), rk(bk.begin(), bk.end());
+            // the level-0 blocks of same-level faces as kernel constants
+            constexpr size_t BB = (size_t)NP * NP;
+            constexpr size_t FST = (size_t)8 * (1 + 2 * NSUB) * 2 * BB;
+            for (size_t i = 0; i < BB; ++i) {
+                (&op.vol[0][0])[i] = rv[i];
+                for (int f = 0; f < NF; ++f)
+                    for (int side = 0; side < 2; ++side) (&op.face[f][side][0][0])[i] = rf[f * FST + side * BB + i];
+            }
+            for (int q = 0; q < NP; ++q) op.wq[q] = R(1);
             MDL_CK(qvol.ensure(rv.size()));
             MDL_CK(qface.ensure(rf.size()));
             MDL_CK(qkelly.ensure(rk.size()));
@@ -797,11 +826,15 @@ public:
             MDL_CK(cudaMemcpy(tcC.p, hc.data(), hc.size() * sizeof(float), cudaMemcpyHostToDevice));
             MDL_CK(cudaFuncSetAttribute((k_tick_tc<DIM, P>), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         tc::SMEM_BYTES));
+            MDL_CK(cudaFuncSetAttribute((k_tick_q23<DIM, P>), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        q23::smem_bytes(256)));
         }
         MDL_CK(dT.ensure(1));
         MDL_CK(dph.ensure(1));
         MDL_CK(cudaMemcpy(dT.p, &T, sizeof(Tables<R>), cudaMemcpyHostToDevice));
         MDL_CK(cudaMemcpy(dph.p, &ph, sizeof(Phys<R>), cudaMemcpyHostToDevice));
+        MDL_CK(dop.ensure(1));
+        MDL_CK(cudaMemcpy(dop.p, &op, sizeof(op), cudaMemcpyHostToDevice));
         MDL_CK(mtab.ensure(hm.size()));
         MDL_CK(cudaMemcpyAsync(mtab.p, hm.data(), hm.size() * sizeof(double), cudaMemcpyHostToDevice, st));
         MDL_CK(class_b.ensure(hcb.size()));
@@ -1117,6 +1150,7 @@ public:
         fs->ta = tick_args(fused_cur);
         fs->T = dT.p;
         fs->ph = dph.p;
+        fs->op = dop.p;
         fs->cls = DIM == 2 ? (P == 1 ? FC_2_1 : FC_2_2) : (P == 1 ? FC_3_1 : FC_3_2);
         fs->shift = 0;
         if (Bout) *Bout = B;

@@ -10,9 +10,9 @@ namespace {
 template <typename R, int DIM, int P>
 __device__ __forceinline__ void fused_range(const FusedSlot<R>& fs, int tick, int lo, int hi) {
     for (int idx = lo + (int)threadIdx.x; idx < hi; idx += (int)blockDim.x) {
-        TickMetaT<DIM, P> m;
+        TickMeta<DIM, P> m;
         tick_fetch<R, DIM, P>(fs.ta.d, idx, m);
-        tick_elem<R, DIM, P>(fs.ta, *fs.T, *fs.ph, tick, m, -1.0);
+        tick_elem<R, DIM, P>(fs.ta, *fs.T, *fs.ph, *static_cast<const OpT<R, DIM, P>*>(fs.op), tick, m, -1.0);
     }
 }
 

@@ -27,6 +27,7 @@ struct FusedSlot {
     TickArgs<R> ta;           // the state set the sweep updates, time step, LTS levels, stimuli
     const Tables<R>* T;       // device copies of the slot's basis tables and physics
     const Phys<R>* ph;
+    const void* op;           // ... and of its operator (OpT of the class)
     int32_t cls;              // FusedClass
     int32_t shift;            // Bmax - B: the slot takes part in global ticks divisible by 2^shift
 };

@@ -22,6 +22,7 @@
 #include <type_traits>
 
 #include "../../include/mdl.h"
+#include "mdl_boxop.cuh"
 #include "mdl_element.cuh"
 
 namespace mdl {
@@ -312,84 +313,6 @@ __device__ __forceinline__ void load_seen(const DevArrays<R>& d, int tick, int B
     load_seen_lv<R, NP, NPS>(d, tick, B, nb, d.lvl[nb], un);
 }
 
-// Residual r = (A u)_e with the neighbours seen at tick `tick`.  All same-level and
-// coarser neighbours are gathered before any face arithmetic (their ids, then their
-// level bytes, then their values), so the dependent loads of the faces overlap;
-// hanging faces (finer neighbours) follow on a separate path.
-template <typename R, int DIM, int P>
-__device__ __forceinline__ void element_residual(const DevArrays<R>& d, const Tables<R>& T,
-                                                 const Phys<R>& ph, int tick, int B, int e,
-                                                 uint32_t inf, int lev, const R* u, R* r) {
-    using S = Shape<DIM, P>;
-    constexpr int NP = S::NP, NF = S::NF, NSUB = S::NSUB, NPS = S::NPS;
-#pragma unroll
-    for (int q = 0; q < NP; ++q) r[q] = R(0);
-    if constexpr (P > 1) {
-        // Q2: one face at a time (holding every neighbour's 27 values would spill)
-        volume_term<R, DIM, P>(T, ph, lev, u, r);
-#pragma unroll
-        for (int f = 0; f < NF; ++f) {
-            const int kind = (inf >> (4 * f)) & 3;
-            if (kind == 0) continue;
-            const int k = f >> 1, s = (f & 1) ? 1 : -1;
-            const int nbi = d.nbr[(size_t)e * NF + f];
-            if (kind != 3) {
-                R un[NP];
-                load_seen<R, NP, NPS>(d, tick, B, nbi, un);
-                const int pos = (inf >> (4 * f + 2)) & 3;
-                face_term<R, DIM, P>(T, ph, k, s, lev, -1, u, kind == 1 ? lev : lev - 1,
-                                     kind == 1 ? -1 : pos, un, lev, r);
-            } else {
-                for (int sb = 0; sb < NSUB; ++sb) {
-                    R un[NP];
-                    load_seen<R, NP, NPS>(d, tick, B, d.hang[nbi + sb], un);
-                    face_term<R, DIM, P>(T, ph, k, s, lev, sb, u, lev + 1, -1, un, lev + 1, r);
-                }
-            }
-        }
-        return;
-    }
-    int nbf[NF], src[NF];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) nbf[f] = d.nbr[(size_t)e * NF + f];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-        const int kind = (inf >> (4 * f)) & 3;
-        src[f] = (kind == 1 || kind == 2) ? nbf[f] : e;
-    }
-    uint8_t lvn[NF];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) lvn[f] = d.lvl[src[f]];
-    R un[NF][NP];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) load_seen_lv<R, NP>(d, tick, B, src[f], lvn[f], un[f]);
-    // Q1: precomputed class blocks, r = A_vol u + sum_f (A_own u + A_nb u_nb)
-    constexpr int NREL = 1 + 2 * NSUB;
-    block_mv<R, NP>(d.qvol + (size_t)lev * NP * NP, u, r);
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-        const int kind = (inf >> (4 * f)) & 3;
-        if (kind == 1 || kind == 2) {
-            const int rel = kind == 1 ? 0 : 1 + ((inf >> (4 * f + 2)) & 3);
-            const R* A = d.qface + ((((size_t)f * 8 + lev) * NREL + rel) * 2) * NP * NP;
-            block_mv<R, NP>(A, u, r);
-            block_mv<R, NP>(A + NP * NP, un[f], r);
-        }
-    }
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-        const int kind = (inf >> (4 * f)) & 3;
-        if (kind != 3) continue;
-        for (int sb = 0; sb < NSUB; ++sb) {
-            R uh[NP];
-            load_seen<R, NP>(d, tick, B, d.hang[nbf[f] + sb], uh);
-            const R* A = d.qface + ((((size_t)f * 8 + lev) * NREL + 1 + NSUB + sb) * 2) * NP * NP;
-            block_mv<R, NP>(A, u, r);
-            block_mv<R, NP>(A + NP * NP, uh, r);
-        }
-    }
-}
-
 // Probe activation check for element e after a step from u (at t_old) to un (t_old + dte).
 // The probes inside the leaf are the root GL nodes a with pfl[lev][a_k] == the leaf's cell
 // in every direction k; a pending probe's values before and after the step are the leaf
@@ -486,13 +409,15 @@ __device__ __forceinline__ double tick_time(const TickArgs<R>& a, int tick) {
 }
 
 // Per-element data that stays fixed during a sweep: the element, its level byte and face
-// info, its face neighbours and (Q1) their level bytes.  A tick reads it before waiting for
+// info, its face neighbours and their level bytes.  A tick reads it before waiting for
 // the previous tick (programmatic dependent launch), so after the wait only the values are
 // loaded, all at once.  (info's probe-pending bit may be cleared by an earlier tick of the
 // sweep; a stale bit only repeats a probe check that finds nothing left to do.)
-template <int NF, bool NB>
+template <int DIM, int P>
 struct TickMeta {
-    static constexpr bool HP = NF == 4;   // 2D: the finer neighbours of hanging faces too
+    static constexpr int NF = 2 * DIM;
+    static constexpr bool HP = DIM == 2;  // 2D: the finer neighbours of hanging faces too
+    static constexpr bool PR = P == 1;    // Q1: the probe lookup too
     int e;
     uint32_t inf;
     uint8_t lv;
@@ -504,24 +429,15 @@ struct TickMeta {
     int rid;
     uint32_t pend;                        // probes of the root with no activation time yet
 };
-// Q2: the neighbours are read face by face inside the residual (holding them would spill)
-template <int NF>
-struct TickMeta<NF, false> {
-    int e;
-    uint32_t inf;
-    uint8_t lv;
-};
-template <int DIM, int P>
-using TickMetaT = TickMeta<2 * DIM, P == 1>;
 
 template <typename R, int DIM, int P>
-__device__ __forceinline__ void tick_fetch(const DevArrays<R>& d, int idx, TickMetaT<DIM, P>& m) {
+__device__ __forceinline__ void tick_fetch(const DevArrays<R>& d, int idx, TickMeta<DIM, P>& m) {
+    using M = TickMeta<DIM, P>;
     constexpr int NF = 2 * DIM;
     m.e = d.order[idx];
     m.lv = d.lvl[m.e];
     m.inf = d.info[m.e];
-    if constexpr (P != 1) {
-    } else if constexpr (DIM == 2) {
+    if constexpr (DIM == 2) {
         const int4 n = *reinterpret_cast<const int4*>(d.nbr + (size_t)m.e * 4);
         m.nbf[0] = n.x; m.nbf[1] = n.y; m.nbf[2] = n.z; m.nbf[3] = n.w;
     } else {
@@ -532,7 +448,7 @@ __device__ __forceinline__ void tick_fetch(const DevArrays<R>& d, int idx, TickM
             m.nbf[f + 1] = n.y;
         }
     }
-    if constexpr (P == 1) {
+    if constexpr (M::PR) {
         m.lc = d.loc[m.e];
         m.rid = d.root[m.e];
         // activation times of the root's probes (only this leaf writes those inside it, at its
@@ -544,62 +460,258 @@ __device__ __forceinline__ void tick_fetch(const DevArrays<R>& d, int idx, TickM
             for (int q = 0; q < NP; ++q)
                 if (isinf(d.lat[(int64_t)m.rid * NP + q])) m.pend |= 1u << q;
         }
-        if constexpr (TickMetaT<DIM, P>::HP) {
-#pragma unroll
-            for (int f = 0; f < NF; ++f) {
-                const bool hanging = ((m.inf >> (4 * f)) & 3) == 3;
-#pragma unroll
-                for (int sb = 0; sb < 2; ++sb) {
-                    m.hg[f][sb] = hanging ? d.hang[m.nbf[f] + sb] : m.e;
-                    m.hgl[f][sb] = d.lvl[m.hg[f][sb]];
-                }
-            }
-        }
+    }
+    if constexpr (M::HP) {
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
-            const int kind = (m.inf >> (4 * f)) & 3;
-            m.lvn[f] = d.lvl[(kind == 1 || kind == 2) ? m.nbf[f] : m.e];
+            const bool hanging = ((m.inf >> (4 * f)) & 3) == 3;
+#pragma unroll
+            for (int sb = 0; sb < 2; ++sb) {
+                m.hg[f][sb] = hanging ? d.hang[m.nbf[f] + sb] : m.e;
+                m.hgl[f][sb] = d.lvl[m.hg[f][sb]];
+            }
+        }
+    }
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        const int kind = (m.inf >> (4 * f)) & 3;
+        m.lvn[f] = d.lvl[(kind == 1 || kind == 2) ? m.nbf[f] : m.e];
+    }
+}
+
+// The row of element nb (level byte lv) that holds its value at tick `tick`; `old` is the row of
+// its step's start and th the interpolation weight when it is mid-interval (th = 0 otherwise).
+template <typename R, int NPS>
+__device__ __forceinline__ const R* seen_row(const DevArrays<R>& d, int tick, int B, int nb, uint8_t lv, const R*& old,
+                                             R& th) {
+    const int sh = B - (lv & 7), par = (lv >> 3) & 1;
+    const int rem = tick & ((1 << sh) - 1);
+    const int nw = par ^ (((tick >> sh) + (rem ? 1 : 0)) & 1);
+    th = R(rem) * pow2_neg<R>(sh);
+    const size_t o = (size_t)nb * NPS;
+    old = (nw ? d.V0 : d.V1) + o;
+    return (nw ? d.V1 : d.V0) + o;
+}
+
+// v = (1 - th) old + th v for a neighbour mid-interval (Alg. 1's linear interpolant).
+template <typename R, int NP, int NPS>
+__device__ __forceinline__ void interp_row(const R* old, R th, R* v) {
+    R so[NP];
+    ld_dofs<R, NP, NPS>(old, so);
+#pragma unroll
+    for (int q = 0; q < NP; ++q) v[q] = so[q] + th * (v[q] - so[q]);
+}
+
+// Q1: r = (A u)_e with the neighbours seen at tick `tick`, from the dense blocks: constants of the
+// kernel for same-level faces (level 0, scaled by 2^((2-d) lev), exact), the class blocks in memory
+// for the others.
+template <typename R, int DIM>
+__device__ __forceinline__ void residual_q1(const DevArrays<R>& d, const Q1Op<R, DIM>& op, int tick, int B,
+                                            const TickMeta<DIM, 1>& m, int lev, const R* u, R* r) {
+    using S = Shape<DIM, 1>;
+    constexpr int NP = S::NP, NF = S::NF, NSUB = S::NSUB, NREL = 1 + 2 * NSUB;
+    R un[NF][NP];
+    const R* old[NF];
+    R th[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        const int kind = (m.inf >> (4 * f)) & 3;
+        const bool use = kind == 1 || kind == 2;
+        ld_vec<R, NP>(seen_row<R, NP>(d, tick, B, use ? m.nbf[f] : m.e, use ? m.lvn[f] : m.lv, old[f], th[f]), un[f]);
+    }
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+        R s = R(0);
+#pragma unroll
+        for (int j = 0; j < NP; ++j) s += op.vol[q][j] * u[j];
+        r[q] = s;
+    }
+    bool irr = false;
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        const int kind = (m.inf >> (4 * f)) & 3;
+        irr = irr || kind >= 2;
+        if (th[f] > R(0)) interp_row<R, NP, NP>(old[f], th[f], un[f]);
+        if (kind == 1) {
+#pragma unroll
+            for (int q = 0; q < NP; ++q) {
+                R s = r[q];
+#pragma unroll
+                for (int j = 0; j < NP; ++j) s += op.face[f][0][q][j] * u[j];
+#pragma unroll
+                for (int j = 0; j < NP; ++j) s += op.face[f][1][q][j] * un[f][j];
+                r[q] = s;
+            }
+        }
+    }
+    if (DIM == 3) {
+        const R sc = pow2_neg<R>(lev);
+#pragma unroll
+        for (int q = 0; q < NP; ++q) r[q] *= sc;
+    }
+    if (!irr) return;
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        const int kind = (m.inf >> (4 * f)) & 3;
+        if (kind < 2) continue;
+        const R* A0 = d.qface + (((size_t)f * 8 + lev) * NREL * 2) * NP * NP;
+        if (kind == 2) {
+            const R* A = A0 + (size_t)(1 + ((m.inf >> (4 * f + 2)) & 3)) * 2 * NP * NP;
+            block_mv<R, NP>(A, u, r);
+            block_mv<R, NP>(A + NP * NP, un[f], r);
+        } else {
+#pragma unroll 1
+            for (int sb = 0; sb < NSUB; ++sb) {
+                R uh[NP];
+                int n;
+                uint8_t lv;
+                if constexpr (TickMeta<DIM, 1>::HP) {
+                    n = sb ? m.hg[f][1] : m.hg[f][0];
+                    lv = sb ? m.hgl[f][1] : m.hgl[f][0];
+                } else {
+                    n = d.hang[m.nbf[f] + sb];
+                    lv = d.lvl[n];
+                }
+                const R* o;
+                R t;
+                ld_vec<R, NP>(seen_row<R, NP>(d, tick, B, n, lv, o, t), uh);
+                if (t > R(0)) interp_row<R, NP, NP>(o, t, uh);
+                const R* A = A0 + (size_t)(1 + NSUB + sb) * 2 * NP * NP;
+                block_mv<R, NP>(A, u, r);
+                block_mv<R, NP>(A + NP * NP, uh, r);
+            }
         }
     }
 }
 
-// Q1 residual r = (A u)_e from the class blocks, with the face neighbours and their level
-// bytes already known: r = A_vol u + sum_f (A_own u + A_nb u_nb); hanging faces after.
-template <typename R, int DIM>
-__device__ __forceinline__ void residual_q1(const DevArrays<R>& d, int tick, int B, const TickMetaT<DIM, 1>& m,
-                                            int lev, const R* u, R* r) {
-    using S = Shape<DIM, 1>;
-    constexpr int NP = S::NP, NF = S::NF, NSUB = S::NSUB, NREL = 1 + 2 * NSUB;
+// rho = (M^-1 A u)_e in level-0 units (times 4^level; see mdl_boxop.cuh) with the neighbours
+// seen at tick `tick`, for 2D Q2 elements: every neighbour row is loaded before the arithmetic.
+template <typename R, int DIM, int P>
+__device__ __forceinline__ void box_residual(const DevArrays<R>& d, const BoxOp<R>& op, int tick, int B,
+                                             const TickMeta<DIM, P>& m, const R* u, R* rho) {
+    using S = Shape<DIM, P>;
+    constexpr int NP = S::NP, NF = S::NF, NT = S::NT, NPS = S::NPS;
+    const uint32_t inf = m.inf;
+    const R c = u[NP / 2];
     R un[NF][NP];
+    const R* old[NF];
+    R th[NF];
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
-        const int kind = (m.inf >> (4 * f)) & 3;
-        load_seen_lv<R, NP>(d, tick, B, (kind == 1 || kind == 2) ? m.nbf[f] : m.e, m.lvn[f], un[f]);
+        const int kind = (inf >> (4 * f)) & 3;
+        const bool use = kind == 1 || kind == 2;
+        ld_dofs<R, NP, NPS>(seen_row<R, NPS>(d, tick, B, use ? m.nbf[f] : m.e, use ? m.lvn[f] : m.lv, old[f], th[f]),
+                            un[f]);
     }
+    R y[NP];
 #pragma unroll
-    for (int q = 0; q < NP; ++q) r[q] = R(0);
-    block_mv<R, NP>(d.qvol + (size_t)lev * NP * NP, u, r);
+    for (int q = 0; q < NP; ++q) y[q] = u[q] - c;
+    box_own<R, DIM, P>(op, y, rho);
+    bool irr = false;
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
-        const int kind = (m.inf >> (4 * f)) & 3;
-        if (kind == 1 || kind == 2) {
-            const int rel = kind == 1 ? 0 : 1 + ((m.inf >> (4 * f + 2)) & 3);
-            const R* A = d.qface + ((((size_t)f * 8 + lev) * NREL + rel) * 2) * NP * NP;
-            block_mv<R, NP>(A, u, r);
-            block_mv<R, NP>(A + NP * NP, un[f], r);
+        const int kind = (inf >> (4 * f)) & 3;
+        irr = irr || kind != 1;
+        if (th[f] > R(0)) interp_row<R, NP, NPS>(old[f], th[f], un[f]);
+#pragma unroll
+        for (int q = 0; q < NP; ++q) un[f][q] -= c;
+        if (kind == 1) {
+            R TN[NT], DN[NT];
+            box_trace<R, DIM, P>(op, f >> 1, 1 - (f & 1), un[f], TN, DN);
+            if (op.cross) {
+                R Xv[NT];
+                box_mixed<R, DIM, P>(op, f >> 1, f & 1, TN, Xv);
+                box_lift<R, DIM, P, true>(op, f >> 1, f & 1, TN, DN, Xv, rho);
+            } else {
+                box_lift<R, DIM, P, false>(op, f >> 1, f & 1, TN, DN, nullptr, rho);
+            }
         }
     }
+    if (!irr) return;
+    // boundary, coarser and finer neighbours
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
-        const int kind = (m.inf >> (4 * f)) & 3;
-        if (kind != 3) continue;
-        for (int sb = 0; sb < NSUB; ++sb) {
-            R uh[NP];
-            if constexpr (TickMetaT<DIM, 1>::HP) load_seen_lv<R, NP>(d, tick, B, m.hg[f][sb], m.hgl[f][sb], uh);
-            else load_seen<R, NP>(d, tick, B, d.hang[m.nbf[f] + sb], uh);
-            const R* A = d.qface + ((((size_t)f * 8 + lev) * NREL + 1 + NSUB + sb) * 2) * NP * NP;
-            block_mv<R, NP>(A, u, r);
-            block_mv<R, NP>(A + NP * NP, uh, r);
+        const int kind = (inf >> (4 * f)) & 3;
+        if (kind == 1) continue;
+        auto nb = [&](int sb, R* v) {
+            if (kind == 2) {
+#pragma unroll
+                for (int q = 0; q < NP; ++q) v[q] = un[f][q];
+                return;
+            }
+            int n;
+            uint8_t lv;
+            if constexpr (TickMeta<DIM, P>::HP) {
+                n = sb ? m.hg[f][1] : m.hg[f][0];
+                lv = sb ? m.hgl[f][1] : m.hgl[f][0];
+            } else {
+                n = d.hang[m.nbf[f] + sb];
+                lv = d.lvl[n];
+            }
+            const R* o;
+            R t;
+            ld_dofs<R, NP, NPS>(seen_row<R, NPS>(d, tick, B, n, lv, o, t), v);
+            if (t > R(0)) interp_row<R, NP, NPS>(o, t, v);
+#pragma unroll
+            for (int q = 0; q < NP; ++q) v[q] -= c;
+        };
+        R TN[NT], DN[NT], Xv[NT];
+        box_face_irregular<R, DIM, P>(op, f >> 1, f & 1, kind, (inf >> (4 * f + 2)) & 3, y, nb, TN, DN, Xv);
+        box_lift<R, DIM, P, true>(op, f >> 1, f & 1, TN, DN, Xv, rho);
+    }
+}
+
+// The same for Q2 3D elements (27 values a row: all six neighbours would spill).  The axis is
+// unrolled, the side a loop: the straight-line form of the whole step is 50 KB of code, which
+// every warp streams through the instruction cache once per element, and waited there for
+// most of its time (8.3 of 15.4 cycles per instruction on a 29k-element block).
+template <typename R>
+__device__ __forceinline__ void box_residual_q23(const DevArrays<R>& d, const BoxOp<R>& op, int tick, int B,
+                                                 const TickMeta<3, 2>& m, const R* u, R* rho) {
+    constexpr int NP = 27, NPS = 28, NT = 9;
+    const uint32_t inf = m.inf;
+    const R c = u[NP / 2];
+    R y[NP];
+#pragma unroll
+    for (int q = 0; q < NP; ++q) y[q] = u[q] - c;
+    box_own<R, 3, 2>(op, y, rho);
+    auto row = [&](int n, uint8_t lv, R* v) {
+        const R* o;
+        R t;
+        ld_dofs<R, NP, NPS>(seen_row<R, NPS>(d, tick, B, n, lv, o, t), v);
+        if (t > R(0)) interp_row<R, NP, NPS>(o, t, v);
+#pragma unroll
+        for (int q = 0; q < NP; ++q) v[q] -= c;
+    };
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+#pragma unroll 1
+        for (int side = 0; side < 2; ++side) {
+            const uint32_t fi = inf >> (8 * k + 4 * side);
+            const int kind = fi & 3;
+            const int nbf = side ? m.nbf[2 * k + 1] : m.nbf[2 * k];
+            const uint8_t lvn = side ? m.lvn[2 * k + 1] : m.lvn[2 * k];
+            R TN[NT], DN[NT];
+            if (kind == 1) {
+                R v[NP];
+                row(nbf, lvn, v);
+                box_trace<R, 3, 2>(op, k, 1 - side, v, TN, DN);
+                if (!op.cross) {
+                    box_lift<R, 3, 2, false>(op, k, side, TN, DN, nullptr, rho);
+                    continue;
+                }
+            }
+            R Xv[NT];
+            if (kind == 1) {
+                box_mixed<R, 3, 2>(op, k, side, TN, Xv);
+            } else {
+                auto nb = [&](int sb, R* v) {
+                    const int n = kind == 2 ? nbf : d.hang[nbf + sb];
+                    row(n, kind == 2 ? lvn : d.lvl[n], v);
+                };
+                box_face_irregular<R, 3, 2>(op, k, side, kind, (fi >> 2) & 3, y, nb, TN, DN, Xv);
+            }
+            box_lift<R, 3, 2, true>(op, k, side, TN, DN, Xv, rho);
         }
     }
 }
@@ -620,6 +732,49 @@ __device__ __forceinline__ void dof_stim(const TickArgs<R>& a, int e, int tick, 
         const R amp = (R)a.stim.amp[s];
         if (on_o) so -= amp;
         if (on_m) sm -= amp;
+    }
+}
+
+// The same for a whole element: bit q of mo[s] (mm[s]) is set where stimulus s acts on node q
+// at the step start (midpoint).  The time windows are tested once per element and stimulus: an
+// FP64 comparison per DOF costs more than the rest of the DOF's step (FP64 is slow on this part).
+struct StimMasks {
+    uint32_t mo[MDL_MAX_STIM], mm[MDL_MAX_STIM];
+    bool any;
+};
+
+template <typename R>
+__device__ __forceinline__ void elem_stim(const TickArgs<R>& a, int e, uint32_t inf, int tick, double dte_d,
+                                          StimMasks& sm) {
+    sm.any = false;
+#pragma unroll
+    for (int s = 0; s < MDL_MAX_STIM; ++s) sm.mo[s] = sm.mm[s] = 0u;
+    if (!(inf & INFO_STIM)) return;
+    const double t_i = tick_time(a, tick);
+    const double t_mid = t_i + 0.5 * dte_d;
+#pragma unroll
+    for (int s = 0; s < MDL_MAX_STIM; ++s) {
+        if (s >= a.stim.n) break;
+        const bool on_o = (a.stim.t0[s] <= t_i) && (t_i < a.stim.t1[s]);
+        const bool on_m = (a.stim.t0[s] <= t_mid) && (t_mid < a.stim.t1[s]);
+        if (!on_o && !on_m) continue;
+        const uint32_t m = a.d.smask[s][e];
+        sm.mo[s] = on_o ? m : 0u;
+        sm.mm[s] = on_m ? m : 0u;
+        sm.any = sm.any || m;
+    }
+}
+
+// Stimulus currents of node q (step start, midpoint).
+template <typename R>
+__device__ __forceinline__ void node_stim(const TickArgs<R>& a, const StimMasks& sm, int q, R& so, R& smd) {
+    so = smd = R(0);
+    if (!sm.any) return;
+#pragma unroll
+    for (int s = 0; s < MDL_MAX_STIM; ++s) {
+        const R amp = (R)a.stim.amp[s];
+        if ((sm.mo[s] >> q) & 1u) so -= amp;
+        if ((sm.mm[s] >> q) & 1u) smd -= amp;
     }
 }
 
@@ -644,101 +799,202 @@ __device__ __forceinline__ R dof_update(const Phys<R>& ph, R Mq, R Minv, int ke,
     return Mq * (dI * dI + dg * dg);
 }
 
-// dof_update for an element without stimulus under the Aliev-Panfilov model (ionic 0) with
-// the exponential state step (integrator 1): the same expressions as ap_iion, ap_g and
-// ap_step_state without their model and integrator branches, and e^x - 1 as a select of both
-// forms, so that the code is straight-line and the items of a thread can interleave.  FIRST:
-// the element's first step of the barrier (ke == 0), which sets Ia and ga to I and g at the
-// step start; otherwise they are inputs.
-template <bool FIRST>
-__device__ __forceinline__ float dof_update_ap(const Phys<float>& ph, float Mq, float Minv, float dte, float u, float w,
-                                               float r, float& Ia, float& ga, float& un, float& wn) {
-    const float I = (ph.k * u * (u - ph.a) * (u - 1.0f) + u * w) * ph.inv_ts;
-    un = u + dte * (-r * Minv - I);
-    const float vinf = -ph.k * u * (u - ph.a - 1.0f);
-    const float den = fmaxf(u + ph.mu2, 1e-6f);
-    const float eps = ph.eps0 + __fdividef(ph.mu1 * w, den);
-    if (FIRST) {
-        Ia = I;
-        ga = eps * (vinf - w) * ph.inv_ts;
-    }
-    const float x = -eps * dte * ph.inv_ts;
-    const float em1_t =
-        x * (1.0f + x * (0.5f + x * (1.0f / 6.0f + x * (1.0f / 24.0f + x * (1.0f / 120.0f + x * (1.0f / 720.0f))))));
-    const float em1_e = expf(x) - 1.0f;
-    wn = w + (w - vinf) * (fabsf(x) < 0.0625f ? em1_t : em1_e);
-    const float Vm = 0.5f * (u + un);
-    const float wm = 0.5f * (w + wn);
-    const float dI = (ph.k * Vm * (Vm - ph.a) * (Vm - 1.0f) + Vm * wm) * ph.inv_ts - Ia;
-    const float vinf_m = -ph.k * Vm * (Vm - ph.a - 1.0f);
-    const float den_m = fmaxf(Vm + ph.mu2, 1e-6f);
-    const float dg = (ph.eps0 + __fdividef(ph.mu1 * wm, den_m)) * (vinf_m - wm) * ph.inv_ts - ga;
-    return Mq * (dI * dI + dg * dg);
-}
+// Constants of the FP32 Aliev-Panfilov step with the time scale folded in.
+struct ApConst {
+    float k, a1, kt, kta, it, eps0, mu1, mu2;
+    __device__ __forceinline__ explicit ApConst(const Phys<float>& ph)
+        : k(ph.k), a1(ph.a + 1.0f), kt(ph.k * ph.inv_ts), kta(ph.k * ph.inv_ts * ph.a), it(ph.inv_ts), eps0(ph.eps0),
+          mu1(ph.mu1), mu2(ph.mu2) {}
+};
 
-// dof_update for DOF q of an element of refinement level lev (mass from the tables).
-template <typename R, int DIM, int P>
-__device__ __forceinline__ R dof_step(const Tables<R>& T, const Phys<R>& ph, int lev, int q, int ke, R dte, R so,
-                                      R sm, R u, R w, R r, R& Ia, R& ga, R& un, R& wn) {
-    constexpr int N1 = P + 1;
-    R Mq = ph.Wvol[lev];
+// dof_update of W DOFs under the Aliev-Panfilov model (ionic 0) with the exponential state step
+// (integrator 1) in FP32: straight-line code, so that the DOFs interleave.  With
+// q = u (u - a - 1): v_inf = -k q and I = u (k (q + a) + w), which shares the cubic's products
+// between I and v_inf; V and w are updated by one addition of their increment, and the midpoints
+// take half of it.  e^x - 1 (x = -eps dt / time scale) is the exponential's Taylor series: through
+// x^4 while every |x| < 2^-7 (truncation below 4e-11 relative; all explicit substeps in practice),
+// else expm1_f32.  first: the elements' first step of the barrier, which sets Ia and ga to I and g
+// at the step start; otherwise they are inputs.  r: M^-1 A u up to the factor sc.  Returns the sum
+// of mq [dI^2 + dg^2].
+template <int W>
+__device__ __forceinline__ float ap_step(const ApConst& c, const bool first, const float* mq, float sc, float dte,
+                                         const float* so, const float* sm, const float* u, const float* w,
+                                         const float* r, float* Ia, float* ga, float* un, float* wn) {
+    float I[W], z[W], x[W], mx = 0.0f;
+    const float xt = -dte * c.it;
 #pragma unroll
-    for (int k = 0; k < DIM; ++k) Mq *= T.w[digit<N1>(q, k)];
-    return dof_update<R>(ph, Mq, ph.Minv[lev][q], ke, dte, so, sm, u, w, r, Ia, ga, un, wn);
+    for (int j = 0; j < W; ++j) {
+        const float q = u[j] * (u[j] - c.a1);
+        z[j] = -c.k * q - w[j];                                      // v_inf - w
+        I[j] = u[j] * (c.kt * q + c.kta + c.it * w[j]) + so[j];
+        const float den = fmaxf(u[j] + c.mu2, 1e-6f);
+        const float eps = c.eps0 + __fdividef(c.mu1 * w[j], den);
+        x[j] = eps * xt;
+        mx = fmaxf(mx, fabsf(x[j]));
+        if (first) {
+            Ia[j] = I[j];
+            ga[j] = eps * z[j] * c.it;
+        }
+    }
+    if (mx < 0.0078125f) {
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+            const float t = x[j];
+            x[j] = t * (1.0f + t * (0.5f + t * (1.0f / 6.0f + t * (1.0f / 24.0f))));
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < W; ++j) x[j] = expm1_f32(x[j]);
+    }
+    float term = 0.0f;
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+        const float du = dte * (-r[j] * sc - I[j]);
+        const float dw = -z[j] * x[j];
+        un[j] = u[j] + du;
+        wn[j] = w[j] + dw;
+        const float Vm = u[j] + 0.5f * du, wm = w[j] + 0.5f * dw;
+        const float q = Vm * (Vm - c.a1);
+        const float dI = Vm * (c.kt * q + c.kta + c.it * wm) + (sm[j] - Ia[j]);
+        const float den = fmaxf(Vm + c.mu2, 1e-6f);
+        const float eps = c.eps0 + __fdividef(c.mu1 * wm, den);
+        const float dg = eps * (-c.k * q - wm) * c.it - ga[j];
+        term += mq[j] * (dI * dI + dg * dg);
+    }
+    return term;
 }
 
-// Pointwise part of one element step (Alg. 1) given the residual r = (A u)_e (dof_step for
-// every DOF); returns the element's RV-T term, vmax = max_q |V_new|.
+// Pointwise part of one element step (Alg. 1) given the residual: Q1 r = (A u)_e (the GL
+// masses of an element are equal), Q2 rho = (M^-1 A u)_e in level-0 units (4^lev scales it); returns the element's RV-T term, vmax = max_q |V_new|.
 template <typename R, int DIM, int P>
-__device__ __forceinline__ R elem_pointwise(const TickArgs<R>& a, const Tables<R>& T, const Phys<R>& ph, int tick,
+__device__ __forceinline__ R elem_pointwise(const TickArgs<R>& a, const Phys<R>& ph, const OpT<R, DIM, P>& op, int tick,
                                             int e, uint32_t inf, int b, int ke, int lev, const R* u, const R* w,
                                             const R* r, R* Ia, R* ga, R* un, R* wn, R& vmax) {
     constexpr int NP = Shape<DIM, P>::NP;
     const double dte_d = a.dte[b];
     const R dte = a.dteR[b];
+    const R sc = P == 1 ? ph.Minv[lev][0] : R(1 << (2 * lev));
     R term = R(0);
     vmax = R(0);
+    StimMasks stm;
+    elem_stim<R>(a, e, inf, tick, dte_d, stm);
     if constexpr (sizeof(R) == 4) {
-        // no stimulus, Aliev-Panfilov, exponential state step: the straight-line update, so
-        // that the element's DOFs interleave
-        if (!(inf & INFO_STIM) && ph.ionic == 0 && ph.integrator == 1) {
-            auto run = [&](auto first) {
-                constexpr bool FIRST = decltype(first)::value;
+        // Aliev-Panfilov, exponential state step: the straight-line update, so that the element's
+        // DOFs interleave
+        if (ph.ionic == 0 && ph.integrator == 1) {
+            R so[NP], smd[NP];
 #pragma unroll
-                for (int q = 0; q < NP; ++q) {
-                    constexpr int N1 = P + 1;
-                    R Mq = ph.Wvol[lev];
+            for (int q = 0; q < NP; ++q) node_stim<R>(a, stm, q, so[q], smd[q]);
+            term = ph.Wvol[lev] * ap_step<NP>(ApConst(ph), ke == 0, op.wq, sc, dte, so, smd, u, w, r, Ia, ga, un, wn);
 #pragma unroll
-                    for (int kk = 0; kk < DIM; ++kk) Mq *= T.w[digit<N1>(q, kk)];
-                    term += dof_update_ap<FIRST>(ph, Mq, ph.Minv[lev][q], dte, u[q], w[q], r[q], Ia[q], ga[q], un[q],
-                                                 wn[q]);
-                    const R av = un[q] < R(0) ? -un[q] : un[q];
-                    vmax = av > vmax ? av : vmax;
-                }
-            };
-            if (ke == 0) run(std::true_type{});
-            else run(std::false_type{});
+            for (int q = 0; q < NP; ++q) vmax = fmaxf(vmax, fabsf(un[q]));
             return term;
         }
     }
 #pragma unroll
     for (int q = 0; q < NP; ++q) {
-        R so = R(0), sm = R(0);
-        if (inf & INFO_STIM) dof_stim<R>(a, e, tick, dte_d, q, so, sm);
-        term += dof_step<R, DIM, P>(T, ph, lev, q, ke, dte, so, sm, u[q], w[q], r[q], Ia[q], ga[q], un[q], wn[q]);
+        R so, smd;
+        node_stim<R>(a, stm, q, so, smd);
+        term += dof_update<R>(ph, ph.Wvol[lev] * op.wq[q], sc, ke, dte, so, smd, u[q], w[q], r[q], Ia[q], ga[q], un[q],
+                              wn[q]);
         const R av = un[q] < R(0) ? -un[q] : un[q];
         vmax = av > vmax ? av : vmax;
     }
     return term;
 }
 
+// Four consecutive values of a row (16-byte vectors; FP64 as two).
+template <typename R>
+__device__ __forceinline__ void ld4(const R* p, R* x) { ld_vec<R, 4>(p, x); }
+template <typename R>
+__device__ __forceinline__ void st4(R* p, const R* x) { st_vec<R, 4>(p, x); }
+
+// Pointwise part of a Q2 3D element step, four DOFs at a time in a loop (unrolled, its code alone
+// is 20 KB): rho in `rw` (28 values, pad 0), the rows of the element streamed with the next four
+// DOFs' loads in flight.  The pad value steps too and stays 0 (its weight is 0).
+template <typename R>
+__device__ __forceinline__ R pointwise_q23(const TickArgs<R>& a, const Phys<R>& ph, const BoxOp<R>& op, int tick, int e,
+                                           uint32_t inf, int b, int ke, int lev, const R* Vc, R* Vd, const R* rw,
+                                           R& vmax) {
+    constexpr int NPS = 28;
+    const DevArrays<R>& d = a.d;
+    const size_t o = (size_t)e * NPS;
+    R* const vp = d.v + o;
+    R* const Ip = d.Ia + o;
+    R* const gp = d.ga + o;
+    const R dte = a.dteR[b], sc = R(1 << (2 * lev)), Wv = ph.Wvol[lev];
+    const bool first = ke == 0, keep = first && b > 0;
+    const bool ap = sizeof(R) == 4 && ph.ionic == 0 && ph.integrator == 1;   // (one for all threads)
+    StimMasks stm;
+    elem_stim<R>(a, e, inf, tick, a.dte[b], stm);
+    R term = R(0);
+    vmax = R(0);
+    R u[4], w[4], Ia[4], ga[4];
+    auto load = [&](int i, R* u_, R* w_, R* I_, R* g_) {
+        ld4<R>(Vc + 4 * i, u_);
+        ld4<R>(vp + 4 * i, w_);
+        if (!first) {
+            ld4<R>(Ip + 4 * i, I_);
+            ld4<R>(gp + 4 * i, g_);
+        }
+    };
+#pragma unroll
+    for (int k = 0; k < 4; ++k) Ia[k] = ga[k] = R(0);
+    load(0, u, w, Ia, ga);
+#pragma unroll 1
+    for (int i = 0; i < 7; ++i) {
+        R u2[4], w2[4], I2[4], g2[4], r[4], un[4], wn[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) I2[k] = g2[k] = R(0);
+        if (i < 6) load(i + 1, u2, w2, I2, g2);
+        else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) u2[k] = w2[k] = R(0);
+        }
+        ld4<R>(rw + 4 * i, r);
+        R so[4], smd[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) node_stim<R>(a, stm, 4 * i + k, so[k], smd[k]);
+        if constexpr (sizeof(R) == 4) {
+            if (ap)
+                term += ap_step<4>(ApConst(ph), first, op.wq + 4 * i, sc, dte, so, smd, u, w, r, Ia, ga, un, wn);
+        }
+        if (!ap) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                term += dof_update<R>(ph, op.wq[4 * i + k], sc, ke, dte, so[k], smd[k], u[k], w[k], r[k], Ia[k],
+                                      ga[k], un[k], wn[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const R av = un[k] < R(0) ? -un[k] : un[k];
+            vmax = av > vmax ? av : vmax;
+        }
+        st4<R>(Vd + 4 * i, un);
+        st4<R>(vp + 4 * i, wn);
+        if (keep) {
+            st4<R>(Ip + 4 * i, Ia);
+            st4<R>(gp + 4 * i, ga);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            u[k] = u2[k];
+            w[k] = w2[k];
+            Ia[k] = I2[k];
+            ga[k] = g2[k];
+        }
+    }
+    return Wv * term;
+}
+
 // One element step of Alg. 1 at tick `tick`: forward Euler on V, exponential/FE step on
 // v, the RV-T accumulation and the element's probe check.
 template <typename R, int DIM, int P>
-__device__ __forceinline__ void tick_elem(const TickArgs<R>& a, const Tables<R>& T, const Phys<R>& ph, int tick,
-                                          const TickMetaT<DIM, P>& m, double t_tick) {
+__device__ __forceinline__ void tick_elem(const TickArgs<R>& a, const Tables<R>& T, const Phys<R>& ph,
+                                          const OpT<R, DIM, P>& op, int tick, const TickMeta<DIM, P>& m,
+                                          double t_tick) {
     using S = Shape<DIM, P>;
-    constexpr int NP = S::NP;
+    constexpr int NP = S::NP, NPS = S::NPS;
     const DevArrays<R>& d = a.d;
     const int e = m.e;
     const uint32_t inf = m.inf;
@@ -746,68 +1002,74 @@ __device__ __forceinline__ void tick_elem(const TickArgs<R>& a, const Tables<R>&
     const int ke = tick >> (a.B - b);
     const int cur = par ^ (ke & 1);
     const int lev = (inf >> 24) & 15;
-    constexpr int NPS = S::NPS;
     const R* Vc = (cur ? d.V1 : d.V0) + (size_t)e * NPS;
     R* Vd = (cur ? d.V0 : d.V1) + (size_t)e * NPS;
     R* vp = d.v + (size_t)e * NPS;
-    // every value this step needs is addressed by now: issue the loads together
-    R u[NP], w[NP], r[NP], Ia[NP], ga[NP];
-    ld_dofs<R, NP, NPS>(Vc, u);
-    ld_dofs<R, NP, NPS>(vp, w);
-    double acc0 = 0.0;
-    if constexpr (P == 1) {
-        if (ke != 0) {
-            ld_dofs<R, NP, NPS>(d.Ia + (size_t)e * NPS, Ia);
-            ld_dofs<R, NP, NPS>(d.ga + (size_t)e * NPS, ga);
-            acc0 = d.acc[e];
-        }
-        residual_q1<R, DIM>(d, tick, a.B, m, lev, u, r);
-    } else {
-        // Q2: the barrier-start terms are loaded after the residual (register pressure)
-        element_residual<R, DIM, P>(d, T, ph, tick, a.B, e, inf, lev, u, r);
-        if (ke != 0) {
-            ld_dofs<R, NP, NPS>(d.Ia + (size_t)e * NPS, Ia);
-            ld_dofs<R, NP, NPS>(d.ga + (size_t)e * NPS, ga);
-            acc0 = d.acc[e];
-        }
-    }
-
-    R un[NP], wn[NP], vmax;
-    const R term = elem_pointwise<R, DIM, P>(a, T, ph, tick, e, inf, b, ke, lev, u, w, r, Ia, ga, un, wn, vmax);
     const double dte_d = a.dte[b];
-    if (ke == 0 && b > 0) {
-        st_dofs<R, NP, NPS>(d.Ia + (size_t)e * NPS, Ia);
-        st_dofs<R, NP, NPS>(d.ga + (size_t)e * NPS, ga);
-    }
-    st_dofs<R, NP, NPS>(Vd, un);
-    st_dofs<R, NP, NPS>(vp, wn);
-    d.acc[e] = acc0 + dte_d * (double)term;
-    if ((inf & INFO_PENDING) && vmax >= ph.lat_gate)
-    {
-        const double tt = t_tick >= 0.0 ? t_tick : tick_time(a, tick);
-        if constexpr (P == 1)
-            lat_check_at<R, DIM, P>(d, T, ph, e, inf, lev, m.lc, m.rid, u, un, tt, dte_d, m.pend, true);
-        else lat_check<R, DIM, P>(d, T, ph, e, inf, lev, u, un, tt, dte_d);
+    const double acc0 = ke != 0 ? d.acc[e] : 0.0;
+    const bool pend = (inf & INFO_PENDING) != 0;
+    R vmax;
+    if constexpr (DIM == 3 && P == 2) {
+        R rl[NPS];                      // rho, read back in a loop: local memory
+        {
+            R u[NP], rho[NP];
+            ld_dofs<R, NP, NPS>(Vc, u);
+            box_residual_q23<R>(d, op, tick, a.B, m, u, rho);
+#pragma unroll
+            for (int q = 0; q < NPS; ++q) rl[q] = q < NP ? rho[q] : R(0);
+        }
+        const R term = pointwise_q23<R>(a, ph, op, tick, e, inf, b, ke, lev, Vc, Vd, rl, vmax);
+        d.acc[e] = acc0 + dte_d * (double)term;
+        if (pend && vmax >= ph.lat_gate)
+            lat_check<R, DIM, P>(d, T, ph, e, inf, lev, Vc, Vd, t_tick >= 0.0 ? t_tick : tick_time(a, tick), dte_d);
+    } else {
+        // every value this step needs is addressed by now: issue the loads together
+        R u[NP], w[NP], r[NP], Ia[NP], ga[NP];
+        ld_dofs<R, NP, NPS>(Vc, u);
+        ld_dofs<R, NP, NPS>(vp, w);
+        if (ke != 0) {
+            ld_dofs<R, NP, NPS>(d.Ia + (size_t)e * NPS, Ia);
+            ld_dofs<R, NP, NPS>(d.ga + (size_t)e * NPS, ga);
+        }
+        if constexpr (P == 1) residual_q1<R, DIM>(d, op, tick, a.B, m, lev, u, r);
+        else box_residual<R, DIM, P>(d, op, tick, a.B, m, u, r);
+        R un[NP], wn[NP];
+        const R term = elem_pointwise<R, DIM, P>(a, ph, op, tick, e, inf, b, ke, lev, u, w, r, Ia, ga, un, wn, vmax);
+        if (ke == 0 && b > 0) {
+            st_dofs<R, NP, NPS>(d.Ia + (size_t)e * NPS, Ia);
+            st_dofs<R, NP, NPS>(d.ga + (size_t)e * NPS, ga);
+        }
+        st_dofs<R, NP, NPS>(Vd, un);
+        st_dofs<R, NP, NPS>(vp, wn);
+        d.acc[e] = acc0 + dte_d * (double)term;
+        if (pend && vmax >= ph.lat_gate) {
+            const double tt = t_tick >= 0.0 ? t_tick : tick_time(a, tick);
+            if constexpr (P == 1)
+                lat_check_at<R, DIM, P>(d, T, ph, e, inf, lev, m.lc, m.rid, u, un, tt, dte_d, m.pend, true);
+            else lat_check<R, DIM, P>(d, T, ph, e, inf, lev, u, un, tt, dte_d);
+        }
     }
 }
 
 // One tick of Alg. 1 over the due elements (a prefix of `order`), for callers that
 // already waited for the previous tick.
 template <typename R, int DIM, int P>
-__device__ __forceinline__ void tick_work(const TickArgs<R>& a, const Tables<R>& T, const Phys<R>& ph, int tick) {
+__device__ __forceinline__ void tick_work(const TickArgs<R>& a, const Tables<R>& T, const Phys<R>& ph,
+                                          const OpT<R, DIM, P>& op, int tick) {
     const int n_act = a.d.meta->nact[tick];
     const double t_tick = -1.0;   // computed where a probe check needs it
     for (int idx = (int)gtid(); idx < n_act; idx += (int)gstride()) {
-        TickMetaT<DIM, P> m;
+        TickMeta<DIM, P> m;
         tick_fetch<R, DIM, P>(a.d, idx, m);
-        tick_elem<R, DIM, P>(a, T, ph, tick, m, t_tick);
+        tick_elem<R, DIM, P>(a, T, ph, op, tick, m, t_tick);
     }
 }
 
 // (The bound's "1" lets the Q1 2D FP32 step keep its 168 registers: under the default heuristic
 // the compiler held it to 128 and spilled 40 bytes, and the C2 sweep ran 11% slower.)
 template <typename R, int DIM, int P>
-__global__ void __launch_bounds__(256, 1) k_tick(const TickArgs<R> a, const Tables<R> T, const Phys<R> ph) {
+__global__ void __launch_bounds__(256, 1) k_tick(
+    const TickArgs<R> a, const Tables<R> T, const Phys<R> ph, const OpT<R, DIM, P> op) {
     // the due count and the first element's metadata are fixed during the sweep: read them
     // while the previous tick drains, then wait for its values (the first tick of a sweep
     // is launched without overlap, after the ordering that writes them)
@@ -815,7 +1077,7 @@ __global__ void __launch_bounds__(256, 1) k_tick(const TickArgs<R> a, const Tabl
     const int n_act = a.d.meta->nact[a.tick];
     const bool bad = a.d.meta->err != 0;
     const int idx0 = (int)gtid();
-    TickMetaT<DIM, P> m;
+    TickMeta<DIM, P> m;
     if (idx0 < n_act) tick_fetch<R, DIM, P>(a.d, idx0, m);
     // the tick's time (FP64, a slow pipe here) only where a probe check may need it
     const double t_tick = (idx0 < n_act && (m.inf & INFO_PENDING)) ? tick_time(a, a.tick) : -1.0;
@@ -823,7 +1085,7 @@ __global__ void __launch_bounds__(256, 1) k_tick(const TickArgs<R> a, const Tabl
     if (bad) return;
     for (int idx = idx0; idx < n_act; idx += (int)gstride()) {
         if (idx != idx0) tick_fetch<R, DIM, P>(a.d, idx, m);
-        tick_elem<R, DIM, P>(a, T, ph, a.tick, m, t_tick);
+        tick_elem<R, DIM, P>(a, T, ph, op, a.tick, m, t_tick);
     }
 }
 
@@ -1244,14 +1506,14 @@ __device__ __forceinline__ void grid_barrier(DevMeta* m, unsigned round, uint32_
 // sized from the occupancy API so that every block is resident.
 template <typename R, int DIM, int P>
 __global__ void __launch_bounds__(256) k_sweep(const TickArgs<R> a, const Tables<R> T, const Phys<R> ph,
-                                              const double* __restrict__ mtab) {
+                                              const OpT<R, DIM, P> op, const double* __restrict__ mtab) {
     using S = Shape<DIM, P>;
     constexpr int NP = S::NP;
     const DevArrays<R>& d = a.d;
     if (d.meta->err) return;             // uniform: nothing below changes err before the end
     const int nt = 1 << a.B;
     for (int i = 0; i < nt; ++i) {
-        tick_work<R, DIM, P>(a, T, ph, i);
+        tick_work<R, DIM, P>(a, T, ph, op, i);
         grid_barrier(d.meta, (unsigned)(i + 1));
     }
     __shared__ double red[256];

@@ -1,9 +1,11 @@
 // mdl_tables.cpp -- basis tables, physics constants and Gershgorin CFL classes (host, FP64).
+#include "mdl_boxop.cuh"
 #include "mdl_tables.h"
 
 #include <math.h>
 
 #include <cmath>
+#include <stddef.h>
 #include <string.h>
 
 #include <vector>
@@ -189,6 +191,74 @@ void convert_phys(const Phys<double>& a, Phys<R>* b) {
     b->lat_gate = (R)a.lat_gate;
 }
 
+void make_boxop(const Tables<double>& T, const Phys<double>& ph, int dim, int p, BoxOp<double>* op) {
+    memset(op, 0, sizeof(*op));
+    const int n = p + 1;
+    for (int i = 0; i < n; ++i) {
+        op->b[0][i] = T.bL[i];
+        op->b[1][i] = T.bR[i];
+        op->dn[0][i] = T.dL[i];
+        op->dn[1][i] = T.dR[i];
+    }
+    for (int a = 0; a < n; ++a)
+        for (int j = 0; j < n; ++j) {
+            op->D1[a][j] = T.D1[a][j];
+            op->Dt[a][j] = T.w[j] * T.D1[j][a] / T.w[a];
+            for (int c = 0; c < 2; ++c) {
+                op->PR[0][c][a][j] = T.Pi[c][a][j];
+                op->PR[1][c][a][j] = 0.5 * T.w[j] * T.Pi[c][j][a] / T.w[a];
+            }
+        }
+    for (int a = 0; a < n; ++a)
+        for (int j = 0; j < n; ++j) {
+            op->C[a][j] = 0.5 * (op->D1[a][j] - op->Dt[a][j]);
+            op->E[a][j] = op->D1[a][j] + op->Dt[a][j];
+        }
+    int np = 1;
+    for (int k = 0; k < dim; ++k) np *= n;
+    for (int q = 0; q < np; ++q) {
+        op->wq[q] = 1.0;
+        int r = q;
+        for (int k = 0; k < dim; ++k, r /= n) op->wq[q] *= T.w[r % n];
+    }
+    for (int k = 0; k < dim; ++k) {
+        const double h2 = ph.h2[0][k], D = ph.D[k][k];
+        op->kap[k] = ph.gamma * D / ph.h[0][k];
+        for (int a = 0; a < n; ++a)
+            for (int j = 0; j < n; ++j)
+                for (int i = 0; i < n; ++i) op->S[k][a][j] += D * h2 * h2 * op->Dt[a][i] * T.D1[i][j];
+        for (int s = 0; s < 2; ++s) {
+            const double sg = s ? 1.0 : -1.0;
+            for (int a = 0; a < n; ++a) {
+                const double be = op->b[s][a] * h2 / T.w[a], da = op->dn[s][a] * h2 * h2 / T.w[a];
+                op->be[k][s][a] = be;
+                op->LT[k][s][a] = -op->kap[k] * be + 0.5 * sg * D * da;
+                op->LD[k][s][a] = -0.5 * sg * D * h2 * be;
+                for (int j = 0; j < n; ++j)
+                    op->S[k][a][j] += (op->kap[k] * be - 0.5 * sg * D * da) * op->b[s][j] -
+                                      0.5 * sg * D * h2 * be * op->dn[s][j];
+            }
+            for (int l = 0; l < dim; ++l) op->XF[k][s][l] = l == k ? 0.0 : -sg * ph.D[k][l] * ph.h2[0][l];
+        }
+        for (int l = 0; l < dim; ++l) op->FK[k][l] = ph.D[k][l] * ph.h2[0][l];
+        for (int l = k + 1; l < dim; ++l) {
+            op->X[k + l - 1] = ph.D[k][l] * h2 * ph.h2[0][l];
+            if (ph.D[k][l] != 0.0) op->cross |= 1 << (k + l - 1);
+        }
+    }
+}
+
+template <typename R>
+void convert_boxop(const BoxOp<double>& a, BoxOp<R>* b) {
+    static_assert(offsetof(BoxOp<R>, cross) % sizeof(R) == 0, "the values come first");
+    const double* x = reinterpret_cast<const double*>(&a);
+    R* y = reinterpret_cast<R*>(b);
+    for (size_t i = 0; i < offsetof(BoxOp<R>, cross) / sizeof(R); ++i) y[i] = (R)x[i];
+    b->cross = a.cross;
+}
+
+template void convert_boxop<float>(const BoxOp<double>&, BoxOp<float>*);
+template void convert_boxop<double>(const BoxOp<double>&, BoxOp<double>*);
 template void convert_tables<float>(const Tables<double>&, Tables<float>*);
 template void convert_tables<double>(const Tables<double>&, Tables<double>*);
 template void convert_phys<float>(const Phys<double>&, Phys<float>*);

@@ -241,7 +241,7 @@ __device__ __forceinline__ float block_row_dot(const float* __restrict__ row, co
 //      row) and the loads of the pointwise step: thread 4 i + p takes DOFs p + 4 m of element i
 //   4  warps 0-3: D row -> scaled residual in shared memory
 //   5  the pointwise step of the thread's DOFs (element metadata read once per thread):
-//      straight-line (dof_update_ap) for a tile without stimulus or padding rows, else
+//      straight-line (ap_step) for a tile without stimulus or padding rows, else
 //      dof_update; the element's RV-T sum and max |V_new| over its four threads by shuffles,
 //      the accumulation and a due probe check; then threads 0..63 build the next tile's
 //      records: per operand slot the row that holds the value the element sees (Alg. 1: a
@@ -604,14 +604,16 @@ __global__ void __launch_bounds__(tc::THREADS, 2)
             auto fast_dofs = [&](auto first) {
                 constexpr bool FIRST = decltype(first)::value;
                 const float dte = sDte[b];
+                const ApConst apc(ph);
 #pragma unroll
                 for (int m = 0; m < NIT; ++m) {
                     const int q = p + 4 * m;
                     if (q < NP) {
                         const float r = sR[i * RST + q] + (irr ? sCorr[i * RST + q] : 0.0f);
                         float un, wn;
-                        term += dof_update_ap<FIRST>(ph, sMq[lev * NP + q], sMinv[lev * NP + q], dte, u[m], w[m], r,
-                                                     Ia[m], ga[m], un, wn);
+                        const float mq = sMq[lev * NP + q], zero = 0.0f;
+                        term += ap_step<1>(apc, FIRST, &mq, sMinv[lev * NP + q], dte, &zero, &zero, u + m, w + m, &r,
+                                           Ia + m, ga + m, &un, &wn);
                         vmax = fmaxf(vmax, fabsf(un));
                         vrow[q] = un;
                         d.v[(size_t)e * NPS + q] = wn;
