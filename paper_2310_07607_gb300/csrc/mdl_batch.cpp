@@ -281,11 +281,10 @@ int fused_issue(mdl_batch* b, const std::vector<int>& run) {
         g.host.clear();
         g.timed = false;
     }
-    // the phases before the sweep, each slot on its own stream; a slot of a group tuned to
-    // own sweeps goes straight on with its sweep
+    // the phases before the sweep, each slot on its own stream; a slot of a group tuned to own
+    // sweeps goes straight on to the end of its barrier
     std::vector<int> Bs(b->slots.size(), 0);
     std::vector<int> begun;
-    std::vector<unsigned char> scratch;
     for (int i : run) {
         mdl_batch::Slot& s = b->slots[i];
         mdl_batch::Group& g = b->groups[s.group];
@@ -293,26 +292,28 @@ int fused_issue(mdl_batch* b, const std::vector<int>& run) {
         // a mapped slot always sweeps on its own and is no member of its group
         const bool alone = s.ctx->impl->is_mapped();
         s.own = alone || (c >= 0 ? c == kOwnCand : g.own);
+        if (s.own && (c < 0 || alone)) {
+            // nothing of the round is shared: the slot's whole barrier in one graph
+            const int rc = s.ctx->impl->fused_whole();
+            if (rc) {
+                s.state = MDL_SLOT_FAILED;
+                s.rc = rc;
+            }
+            if (!alone) g.members.push_back(i);
+            continue;
+        }
         const size_t bytes = mdl::fused_slot_bytes(g.precision);
         const size_t off = g.host.size();
-        unsigned char* rec;
-        if (alone) {
-            scratch.resize(bytes);
-            rec = scratch.data();
-        } else {
-            g.host.resize(off + bytes);
-            rec = g.host.data() + off;
-        }
-        int rc = s.ctx->impl->fused_begin(rec, &Bs[i]);
-        if (!rc && s.own && (c < 0 || alone)) rc = s.ctx->impl->fused_own_sweep();
+        g.host.resize(off + bytes);
+        const int rc = s.ctx->impl->fused_begin(g.host.data() + off, &Bs[i]);
         if (rc) {
-            if (!alone) g.host.resize(off);
+            g.host.resize(off);
             s.state = MDL_SLOT_FAILED;
             s.rc = rc;
             continue;
         }
         MDL_BCK(cudaEventRecord(b->sev[i], (cudaStream_t)s.ctx->impl->stream_handle()));
-        if (!alone) g.members.push_back(i);
+        g.members.push_back(i);
         begun.push_back(i);
     }
     // per (precision, class) group, on the group's own stream (the groups' sweeps overlap):

@@ -51,6 +51,9 @@ public:
     virtual int fused_begin(void* slot_record, int* B) = 0;
     virtual int fused_own_sweep() = 0;
     virtual int fused_finish() = 0;
+    // A whole round of a slot that sweeps on its own: every phase of one barrier on its stream (in
+    // place of fused_begin .. fused_finish).
+    virtual int fused_whole() = 0;
     virtual bool replaying() const = 0;
     // A mapped (curved) geometry: its sweep is always its own (the fused kernel has box
     // elements only).

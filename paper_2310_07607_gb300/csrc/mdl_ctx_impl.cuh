@@ -5,11 +5,10 @@
 // (indicator / adaptation + levels + ordering / sweep / epilogue); element counts, due
 // counts per tick, the barrier counter and errors live in device memory (DevMeta), so
 // the host never waits inside a barrier:
-//   [AMR]  k_eta_s, k_amr_mark, k_amr_close x max_refine, k_amr_family, k_scan_blocks,
-//          k_scan_top (commit), k_scan_emit (coordinates into the other state set),
-//          k_leaf_keys + k_mesh_tables + k_lat_refresh (in place, only if the mesh changed),
-//          k_transfer (state into the other set)
-//   levels k_levels_count, k_order_top, k_order_scatter
+//   [AMR]  k_eta_s (with the refinement marks), k_scan_blocks, k_scan_top (commit), k_scan_emit (coordinates
+//          into the other state set), k_mesh_tables (in place, only if the mesh changed),
+//          k_transfer (state into the other set, levels)
+//   levels k_levels_count (without adaptation), k_order_top, k_order_scatter
 //   sweep  2^B launches of k_tick (each reads its due count from DevMeta)
 //   end    k_epilogue (eta^t, parities, int V by a last-block reduction, counters)
 // The state (V slots, v, eta^t, levels, coordinates) is double-buffered across an
@@ -114,6 +113,7 @@ class Ctx : public CtxBase {
     Tables<R> T{};
     Phys<R> ph{};
     OpT<R, DIM, P> op{};
+    EpiWeights epiw{};
     Grid grid_{};
     StimBoxes sboxes{};
     StimArgs stim{};
@@ -166,11 +166,13 @@ class Ctx : public CtxBase {
     };
     std::vector<EvSet> pending_ev;
     mdl_stats stats{};
-    // captured phase graphs, per phase and state set (an adapting barrier swaps sets)
-    cudaGraphExec_t gexec[4][2] = {};
-    int64_t gcap[4][2] = {{-1, -1}, {-1, -1}, {-1, -1}, {-1, -1}};
-    int64_t glaunch[4][2] = {};
-    int64_t gticks[4][2] = {};
+    // captured graphs of consecutive phases, per first and last phase and state set (an adapting
+    // barrier swaps sets)
+    struct PhaseGraph {
+        cudaGraphExec_t exec = nullptr;
+        int64_t cap = -1, launches = 0, ticks = 0;
+    };
+    PhaseGraph graphs[4][4][2];
     bool use_graphs = true;
     int tick_threads = 128, tick_bpsm = 16;   // sweep launch shape
     bool coop_sweep = false;                  // ticks + epilogue in one cooperative launch
@@ -211,9 +213,18 @@ class Ctx : public CtxBase {
     }
 
     int persistent_blocks(int threads) const {
-        const int64_t need = div_up(std::max<int64_t>(cap, 1), threads);
+        const int64_t need = div_up(sweep_elems(), threads);
         return (int)std::min<int64_t>(need, (int64_t)nsm * (2048 / threads));
     }
+
+    // Threads per block of a sweep over n threads of work: halved (to a warp) while the mesh has
+    // fewer blocks than the chip SMs, so that a small one spreads over more of them.
+    int spread_threads(int64_t n, int threads) const {
+        while (threads > 32 && div_up(n, threads) < nsm) threads /= 2;
+        return threads;
+    }
+    // Elements that a launch is sized for: the mesh's, or the capacity where it adapts.
+    int64_t sweep_elems() const { return std::max<int64_t>(pb.amr_enabled ? cap : ne, 1); }
 
     static constexpr bool tensor_capable = std::is_same<R, float>::value && DIM == 3 && P == 2;
 
@@ -270,6 +281,9 @@ class Ctx : public CtxBase {
         return MDL_OK;
     }
 
+    // Column stride of the ordering's counts: the blocks, in whole groups of 8 (a lane's vector).
+    static int ord_stride(int64_t c) { return (div_up(c, ORD_THREADS) + 7) / 8 * 8; }
+
     int alloc_shared(int64_t c) {
         MDL_CK(Ia.ensure((size_t)c * NPS));
         MDL_CK(ga.ensure((size_t)c * NPS));
@@ -278,13 +292,13 @@ class Ctx : public CtxBase {
         MDL_CK(r.ensure(c));
         MDL_CK(c0.ensure(c));
         MDL_CK(bsum.ensure(div_up(c, SCAN_CHUNK) + 1));
-        MDL_CK(bcnt.ensure((size_t)(div_up(c, ORD_THREADS) + 1) * 8 + 8));
+        MDL_CK(bcnt.ensure((size_t)ORD_KEYS * (ord_stride(c) + 1)));
         MDL_CK(pkind.ensure(c));
         MDL_CK(pbits.ensure(c));
         MDL_CK(psrc.ensure(c));
         if (mapped) MDL_CK(ftodo.ensure(c));
         MDL_CK(partial.ensure((size_t)nsm * 16 + 1024));
-        return MDL_OK;
+        return clear_marks();
     }
 
     template <class T2>
@@ -350,12 +364,13 @@ class Ctx : public CtxBase {
     // unless forced, only when this barrier's adaptation changed the mesh.
     int build_tables(int s, int force) {
         Set& x = sets[s];
-        const int gb = persistent_blocks(256);
-        MDL_CK(launch_k((k_leaf_keys<DIM>), persistent_blocks(256), 256, x.coord.p, lkey.p, grid_, meta.p, force));
-        MDL_LAUNCHED();
+        if (force) {   // (an adaptation writes the keys of its new leaves)
+            MDL_CK(launch_k((k_leaf_keys<DIM>), persistent_blocks(256), 256, x.coord.p, lkey.p, grid_, meta.p));
+            MDL_LAUNCHED();
+        }
         MDL_CK(launch_k((k_mesh_tables<R, DIM, P>), persistent_blocks(128), 128, 
             x.coord.p, lkey.p, grid_, info.p, nbr.p, hang.p, root.p, loc.p, bcfl.p, class_b.p,
-            smask[0].p, smask[1].p, smask[2].p, smask[3].p, sboxes, phd, meta.p, force));
+            smask[0].p, smask[1].p, smask[2].p, smask[3].p, sboxes, phd, T, lat.p, meta.p, force));
         MDL_LAUNCHED();
         return MDL_OK;
     }
@@ -396,6 +411,7 @@ class Ctx : public CtxBase {
         MDL_CK(cudaMemsetAsync(x.eta_t.p, 0, n * sizeof(double), st));
         MDL_CK(cudaMemsetAsync(x.lvl.p, 0, n, st));
         MDL_CK(cudaMemsetAsync(eta_s.p, 0, n * sizeof(double), st));
+        if (int rm = clear_marks()) return rm;
         k_fill_inf<<<div_up(n_probe, 256), 256, 0, st>>>(lat.p, n_probe);
         MDL_LAUNCHED();
         k_lat_refresh<R, DIM, P><<<persistent_blocks(128), 128, 0, st>>>(arrays(cs), T, ph, (double)nbar * dt, 0, 1);
@@ -423,38 +439,84 @@ class Ctx : public CtxBase {
     //   0 indicator (k_eta_s), 1 adaptation + levels + ordering, 2 sweep ticks, 3 epilogue.
     // Phase 0 only runs with adaptation and no replayed eta^s.  No host synchronisation.
     static constexpr int NPHASE = 4;
+    cudaError_t launch_eta(int o) {
+        const int g128 = persistent_blocks(128);
+        if constexpr (tensor_capable) {
+            const int smem = q23::eta_smem_bytes(128);
+            int occ = 0;
+            cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_eta_q23<DIM, P>, 128, smem);
+            if (e != cudaSuccess) return e;
+            return launch_kxs(pdl, (size_t)smem, (k_eta_q23<DIM, P>), std::min(g128, nsm * std::max(1, occ)), 128, arrays(o),
+                              T, ph, op, mark_args());
+        } else if constexpr (P == 2) {
+            return launch_k((k_eta_s_q2<R, DIM>), g128, 128, arrays(o), T, ph, op, mark_args());
+        } else {
+            return launch_k((k_eta_s<R, DIM, P>), g128, 128, arrays(o), T, ph, mark_args());
+        }
+    }
+
+    MarkArgs mark_args() const { return MarkArgs{pb.amr_enabled ? r.p : nullptr, pb.tau_refine, pb.max_refine}; }
+
+    // Refinement marks are 0 between barriers; a barrier that stopped part way may have left some.
+    int clear_marks() {
+        if (r.p) MDL_CK(cudaMemsetAsync(r.p, 0, r.cap, st));
+        return MDL_OK;
+    }
 
     int launch_phase(int ph_, int o) {
         const int g256 = persistent_blocks(256), g128 = persistent_blocks(128);
         if (ph_ == 0) {
-            if (mapped) MDL_CK(launch_k((k_eta_s_mapped<R, DIM, P>), g128, 128, arrays(o), T));
-            else MDL_CK(launch_k((k_eta_s<R, DIM, P>), g128, 128, arrays(o), T, ph));
+            if (mapped) MDL_CK(launch_k((k_eta_s_mapped<R, DIM, P>), g128, 128, arrays(o), T, mark_args()));
+            else MDL_CK(launch_eta(o));
             MDL_LAUNCHED();
             return MDL_OK;
         }
         if (ph_ == 1) {
             int cur = o;
+            const int nob = div_up(cap, ORD_THREADS);
+            LevelArgs la{};
+            la.ovr = ovr_levels ? lvl_ovr.p : nullptr;
+            la.eta_ovr = ovr_eta_t ? eta_t_ovr.p : nullptr;
+            la.tau_cell = pb.tau_cell;
+            if (pb.dt_bar_cell > 0) {
+                la.bcell = b_from_bound(dt, pb.dt_bar_cell);
+                if (la.bcell < 0) la.bcell = 15;
+            }
+            la.B = B;
+            la.lts = pb.lts_enabled;
+            la.bcnt = bcnt.p;
+            la.stride = ord_stride(cap);
+            // irregular: a face that is not a same-level interior one; curved elements skip their
+            // boundary faces, so there a coarser or finer neighbour.  Only where such a face costs
+            // a multiple of a same-level one: for 3D Q2 (3D slab sweep 5.37 -> 5.01 ms) and curved
+            // meshes (adapting FP64 shell 0.88 -> 0.80 ms); Q1 and 2D sweeps lose as much by the
+            // longer warps of irregular elements as they gain (3D Q1 slab 27.8 -> 32.1 us).
+            const uint32_t all = DIM == 2 ? 0x1111u : 0x111111u;
+            if (mapped) la.fmask = 2u * all;
+            else if (DIM == 3 && P == 2) {
+                la.fmask = 3u * all;
+                la.fsame = all;
+            }
             if (pb.amr_enabled) {
                 const int n = o ^ 1;
                 Set& so = sets[o];
                 Set& sn = sets[n];
-                MDL_CK(launch_k((k_amr_mark<DIM>), g256, 256, so.coord.p, eta_s.p, r.p, c0.p, meta.p, pb.tau_refine,
-                                                      pb.max_refine));
-                MDL_LAUNCHED();
-                for (int i = 0; i < pb.max_refine; ++i) {
+                if (ovr_eta_s) {
+                    MDL_CK(launch_k((k_amr_mark<DIM>), g256, 256, info.p, nbr.p, eta_s.p, meta.p, mark_args()));
+                    MDL_LAUNCHED();
+                }
+                for (int i = MARK_CHAIN; i < pb.max_refine - 1; ++i) {
                     MDL_CK(launch_k((k_amr_close<DIM>), g256, 256, info.p, nbr.p, r.p, meta.p));
                     MDL_LAUNCHED();
                 }
-                MDL_CK(launch_k((k_amr_family<DIM>), g256, 256, so.coord.p, info.p, nbr.p, eta_s.p, r.p, c0.p, meta.p,
-                                                        pb.tau_coarsen));
-                MDL_LAUNCHED();
                 const int nsb = div_up(cap, SCAN_CHUNK);
-                MDL_CK(launch_k((k_scan_blocks<DIM>), nsb, SCAN_THREADS, so.coord.p, r.p, c0.p, bsum.p, meta.p));
+                MDL_CK(launch_k((k_scan_blocks<DIM>), nsb, SCAN_THREADS, so.coord.p, info.p, nbr.p, eta_s.p, r.p, c0.p,
+                                bsum.p, meta.p, pb.tau_coarsen));
                 MDL_LAUNCHED();
                 MDL_CK(launch_k((k_scan_top), 1, 1024, bsum.p, meta.p, cap));
                 MDL_LAUNCHED();
                 MDL_CK(launch_k((k_scan_emit<DIM>), nsb, SCAN_THREADS, so.coord.p, r.p, c0.p, bsum.p, sn.coord.p,
-                                                               pkind.p, psrc.p, pbits.p, meta.p));
+                                lkey.p, grid_, pkind.p, psrc.p, pbits.p, meta.p));
                 MDL_LAUNCHED();
                 DevArrays<R> od = arrays(o);
                 int rc = build_tables(n, 0);
@@ -474,25 +536,17 @@ class Ctx : public CtxBase {
                                     (const int32_t*)ftodo.p, meta.p));
                     MDL_LAUNCHED();
                 }
-                MDL_CK(launch_k((k_transfer<R, DIM, P>), g128, 128, od, arrays(n), pkind.p, psrc.p, pbits.p, T));
-                MDL_LAUNCHED();
-                MDL_CK(launch_k((k_lat_refresh<R, DIM, P>), g128, 128, arrays(n), T, ph, 0.0, 0, 0));
+                la.r = r.p;
+                MDL_CK(launch_k((k_transfer<R, DIM, P>), nob, ORD_THREADS, od, arrays(n), pkind.p, psrc.p, pbits.p, T, la));
                 MDL_LAUNCHED();
                 cur = n;
+            } else {
+                MDL_CK(launch_k((k_levels_count<R>), nob, ORD_THREADS, arrays(cur), la));
+                MDL_LAUNCHED();
             }
-            int bcell = 0;
-            if (pb.dt_bar_cell > 0) {
-                bcell = b_from_bound(dt, pb.dt_bar_cell);
-                if (bcell < 0) bcell = 15;
-            }
-            const double* et = ovr_eta_t ? eta_t_ovr.p : sets[cur].eta_t.p;
-            const int nob = div_up(cap, ORD_THREADS);
-            MDL_CK(launch_k((k_levels_count<R>), nob, ORD_THREADS, arrays(cur), ovr_levels ? lvl_ovr.p : nullptr, et,
-                                                           pb.tau_cell, bcell, B, pb.lts_enabled, bcnt.p));
+            MDL_CK(launch_k((k_order_top), 1, 1024, bcnt.p, la.stride, meta.p, B));
             MDL_LAUNCHED();
-            MDL_CK(launch_k((k_order_top), 1, 1024, bcnt.p, meta.p, B));
-            MDL_LAUNCHED();
-            MDL_CK(launch_k((k_order_scatter), nob, ORD_THREADS, sets[cur].lvl.p, bcnt.p, order.p, meta.p));
+            MDL_CK(launch_k((k_order_scatter), nob, ORD_THREADS, sets[cur].lvl.p, bcnt.p, la.stride, order.p, meta.p));
             MDL_LAUNCHED();
             return MDL_OK;
         }
@@ -520,18 +574,20 @@ class Ctx : public CtxBase {
                 return MDL_OK;
             }
             if (mapped) {
-                const int gm = (int)std::min<int64_t>(div_up(std::max<int64_t>(cap, 1), 128), (int64_t)nsm * 16);
+                const int tm = spread_threads(sweep_elems(), 128);
+                const int gm = (int)std::min<int64_t>(div_up(sweep_elems(), tm), (int64_t)nsm * (2048 / tm));
                 for (int i = 0; i < nt; ++i) {
                     ta.tick = i;
-                    MDL_CK(launch_kx(pdl && i > 0, (k_tick_mapped<R, DIM, P>), gm, 128, ta, T, ph));
+                    MDL_CK(launch_kx(pdl && i > 0, (k_tick_mapped<R, DIM, P>), gm, tm, ta, T, ph));
                     MDL_LAUNCHED();
                     stats.tick_launches++;
                 }
                 return MDL_OK;
             }
             const int lanes = (P == 1 && group_tick) ? NP : 1;
-            const int gt = (int)std::min<int64_t>(div_up(std::max<int64_t>(cap, 1) * lanes, tick_threads),
-                                                  (int64_t)nsm * tick_bpsm);
+            const int tt = lanes > 1 ? tick_threads : spread_threads(sweep_elems(), tick_threads);
+            const int gt = (int)std::min<int64_t>(div_up(sweep_elems() * lanes, tt),
+                                                  (int64_t)nsm * tick_bpsm * (tick_threads / tt));
             if constexpr (tensor_capable) {
                 if (tensor_tick) {
                     // persistent: two blocks per SM walk the tiles of 64 due elements; no more
@@ -551,13 +607,13 @@ class Ctx : public CtxBase {
             }
             if constexpr (tensor_capable) {
                 // resident blocks only: each walks its due elements, fetching metadata a step ahead
-                const int smem = q23::smem_bytes(tick_threads);
+                const int smem = q23::smem_bytes(tt);
                 int occ = 0;
-                MDL_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tick_q23<DIM, P>, tick_threads, smem));
+                MDL_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tick_q23<DIM, P>, tt, smem));
                 const int gq = std::min(gt, nsm * std::max(1, occ));
                 for (int i = 0; i < nt; ++i) {
                     ta.tick = i;
-                    MDL_CK(launch_kxs(pdl && i > 0, (size_t)smem, (k_tick_q23<DIM, P>), gq, tick_threads, ta, T, ph, op));
+                    MDL_CK(launch_kxs(pdl && i > 0, (size_t)smem, (k_tick_q23<DIM, P>), gq, tt, ta, T, ph, op));
                     MDL_LAUNCHED();
                     stats.tick_launches++;
                 }
@@ -566,10 +622,10 @@ class Ctx : public CtxBase {
             for (int i = 0; i < nt; ++i) {
                 ta.tick = i;
                 if constexpr (P == 1) {
-                    if (group_tick) MDL_CK(launch_k((k_tick_group<R, DIM>), gt, tick_threads, ta, ph, T));
-                    else MDL_CK(launch_kx(pdl && i > 0, (k_tick<R, DIM, P>), gt, tick_threads, ta, T, ph, op));
+                    if (group_tick) MDL_CK(launch_kx(pdl && i > 0, (k_tick_group<R, DIM>), gt, tt, ta, ph, T));
+                    else MDL_CK(launch_kx(pdl && i > 0, (k_tick<R, DIM, P>), gt, tt, ta, T, ph, op));
                 } else {
-                    MDL_CK(launch_kx(pdl && i > 0, (k_tick<R, DIM, P>), gt, tick_threads, ta, T, ph, op));
+                    MDL_CK(launch_kx(pdl && i > 0, (k_tick<R, DIM, P>), gt, tt, ta, T, ph, op));
                 }
                 MDL_LAUNCHED();
                 stats.tick_launches++;
@@ -579,7 +635,7 @@ class Ctx : public CtxBase {
         {
             int ex = 0;
             const double fr = frexp(dt, &ex);
-            MDL_CK(launch_k((k_epilogue<R, DIM, P>), g256, 256, arrays(o), mapped ? sets[o].mq.p : mtab.p, dt,
+            MDL_CK(launch_k((k_epilogue<R, DIM, P>), g256, 256, arrays(o), mapped ? sets[o].mq.p : mtab.p, epiw, dt,
                             1.0 / dt, fr == 0.5 ? 1 : 0, mapped ? 1 : 0));
         }
         MDL_LAUNCHED();
@@ -601,70 +657,87 @@ class Ctx : public CtxBase {
         return ta;
     }
 
-    // Run phase ph_ on set o: replay its captured graph (capturing it first) unless inputs
-    // are replayed this barrier, in which case launch directly.
-    int run_phase(int ph_, int o, bool direct) {
-        if (direct || !use_graphs) return launch_phase(ph_, o);
-        cudaGraphExec_t& ge = gexec[ph_][o];
-        if (!ge || gcap[ph_][o] != cap) {
-            if (ge) cudaGraphExecDestroy(ge);
-            ge = nullptr;
+    // The state set of phase ph_ of a barrier that starts on set o.
+    int phase_set(int ph_, int o) const { return ph_ >= 2 && pb.amr_enabled ? (o ^ 1) : o; }
+
+    // Run phases p0 .. p1 of the barrier that starts on set o: replay their captured graph
+    // (capturing it first) unless inputs are replayed this barrier, in which case launch directly.
+    int run_phases(int p0, int p1, int o, bool direct) {
+        auto launch_all = [&]() {
+            for (int p = p0; p <= p1; ++p)
+                if (int rc = launch_phase(p, phase_set(p, o))) return rc;
+            return (int)MDL_OK;
+        };
+        if (direct || !use_graphs) return launch_all();
+        PhaseGraph& g = graphs[p0][p1][o];
+        if (!g.exec || g.cap != cap) {
+            if (g.exec) cudaGraphExecDestroy(g.exec);
+            g.exec = nullptr;
             const int64_t kl0 = stats.kernel_launches, tl0 = stats.tick_launches;
             cudaGraph_t graph;
             MDL_CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-            int rc = launch_phase(ph_, o);
+            int rc = launch_all();
             cudaError_t ec = cudaStreamEndCapture(st, &graph);
             if (rc) {
                 if (ec == cudaSuccess) cudaGraphDestroy(graph);
                 return rc;
             }
             MDL_CK(ec);
-            ec = cudaGraphInstantiate(&ge, graph, 0);
+            ec = cudaGraphInstantiate(&g.exec, graph, 0);
             cudaGraphDestroy(graph);
             MDL_CK(ec);
-            glaunch[ph_][o] = stats.kernel_launches - kl0;
-            gticks[ph_][o] = stats.tick_launches - tl0;
+            g.launches = stats.kernel_launches - kl0;
+            g.ticks = stats.tick_launches - tl0;
             stats.kernel_launches = kl0;
             stats.tick_launches = tl0;
-            gcap[ph_][o] = cap;
+            g.cap = cap;
         }
-        MDL_CK(cudaGraphLaunch(ge, st));
-        stats.kernel_launches += glaunch[ph_][o];
-        stats.tick_launches += gticks[ph_][o];
+        MDL_CK(cudaGraphLaunch(g.exec, st));
+        stats.kernel_launches += g.launches;
+        stats.tick_launches += g.ticks;
         return MDL_OK;
     }
 
-    // One barrier step; events around the indicator and the sweep when timing.
+    // The first phase of a barrier: the spatial indicator, for the adaptation and on a mapped mesh
+    // that does not adapt as the barrier's diagnostic; none where it is replayed.
+    int first_phase() const { return (pb.amr_enabled || mapped) && !ovr_eta_s ? 0 : 1; }
+    // The last one: the cooperative sweep runs the epilogue itself.
+    int last_phase() const { return coop_sweep ? 2 : 3; }
+
+    // One barrier step: one graph, or with timing a graph per phase with events around the
+    // indicator and the sweep.
     int run_barrier() {
         const bool direct = ovr_levels || ovr_eta_s || ovr_eta_t;
-        const int o = cs;
+        const int o = cs, p0 = first_phase(), p1 = last_phase();
         int rc;
-        cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr, e3 = nullptr;
-        // the spatial indicator: for the adaptation, and on a mapped mesh (which does not
-        // adapt) as the barrier's diagnostic
-        if ((pb.amr_enabled || mapped) && !ovr_eta_s) {
-            if (timing && (e2 = next_event())) MDL_CK(cudaEventRecord(e2, st));
-            if ((rc = run_phase(0, o, direct))) return rc;
-            if (timing && (e3 = next_event())) MDL_CK(cudaEventRecord(e3, st));
+        if (!timing) {
+            if ((rc = run_phases(p0, p1, o, direct))) return rc;
+            cs = phase_set(p1, o);
+            return MDL_OK;
         }
-        if ((rc = run_phase(1, o, direct))) return rc;
-        const int cur = pb.amr_enabled ? (o ^ 1) : o;
-        if (timing && (e0 = next_event())) MDL_CK(cudaEventRecord(e0, st));
-        if ((rc = run_phase(2, cur, direct))) return rc;
-        if (timing && (e1 = next_event())) MDL_CK(cudaEventRecord(e1, st));
-        if (!coop_sweep && (rc = run_phase(3, cur, direct))) return rc;
-        if (timing) pending_ev.push_back({e0, e1, e2, e3});
-        cs = cur;
+        cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr, e3 = nullptr;
+        if (p0 == 0) {
+            if ((e2 = next_event())) MDL_CK(cudaEventRecord(e2, st));
+            if ((rc = run_phases(0, 0, o, direct))) return rc;
+            if ((e3 = next_event())) MDL_CK(cudaEventRecord(e3, st));
+        }
+        if ((rc = run_phases(1, 1, o, direct))) return rc;
+        if ((e0 = next_event())) MDL_CK(cudaEventRecord(e0, st));
+        if ((rc = run_phases(2, 2, o, direct))) return rc;
+        if ((e1 = next_event())) MDL_CK(cudaEventRecord(e1, st));
+        if (p1 == 3 && (rc = run_phases(3, 3, o, direct))) return rc;
+        pending_ev.push_back({e0, e1, e2, e3});
+        cs = phase_set(p1, o);
         return MDL_OK;
     }
 
     void drop_graphs() {
-        for (int p = 0; p < NPHASE; ++p)
-            for (int i = 0; i < 2; ++i) {
-                if (gexec[p][i]) cudaGraphExecDestroy(gexec[p][i]);
-                gexec[p][i] = nullptr;
-                gcap[p][i] = -1;
-            }
+        for (auto& a : graphs)
+            for (auto& b : a)
+                for (auto& g : b) {
+                    if (g.exec) cudaGraphExecDestroy(g.exec);
+                    g = PhaseGraph{};
+                }
     }
 
     void collect_timing() {
@@ -780,6 +853,13 @@ public:
                 }
             }
         }
+        for (int q = 0; q < NP; ++q) {
+            double w = 1.0;
+            for (int k = 0; k < DIM; ++k) w *= Td.w[digit<N1>(q, k)];
+            epiw.wh[q] = (float)w;
+            epiw.wl[q] = (float)(w - (double)epiw.wh[q]);
+        }
+        epiw.w0 = phd.Wvol[0];
         std::vector<double> hm(8 * NP);
         for (int l = 0; l < 8; ++l)
             for (int q = 0; q < NP; ++q) {
@@ -828,6 +908,8 @@ public:
                                         tc::SMEM_BYTES));
             MDL_CK(cudaFuncSetAttribute((k_tick_q23<DIM, P>), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         q23::smem_bytes(256)));
+            MDL_CK(cudaFuncSetAttribute((k_eta_q23<DIM, P>), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        q23::eta_smem_bytes(128)));
         }
         MDL_CK(dT.ensure(1));
         MDL_CK(dph.ensure(1));
@@ -990,6 +1072,7 @@ public:
             done += nbar - start;
             if (nbar > start) ovr_levels = ovr_eta_s = ovr_eta_t = false;   // consumed by a completed barrier
             const unsigned e = hmeta->err;
+            if (e && (rc = clear_marks())) return rc;
             if (e & ERR_CAPACITY) {
                 if (++retries > 8) {
                     err = "element capacity could not be grown";
@@ -1055,6 +1138,7 @@ public:
         if (done > 0) ovr_levels = ovr_eta_s = ovr_eta_t = false;
         stats.barriers = nbar;
         const unsigned e = hmeta->err;
+        if (e && (rc = clear_marks())) return rc;
         if (e & ERR_CAPACITY) {
             rc = grow(hmeta->need);
             if (rc) return rc;
@@ -1143,9 +1227,8 @@ public:
         fused_own = false;
         const int o = cs;
         int rc;
-        if ((pb.amr_enabled || mapped) && !ovr_eta_s && (rc = run_phase(0, o, direct))) return rc;
-        if ((rc = run_phase(1, o, direct))) return rc;
-        fused_cur = pb.amr_enabled ? (o ^ 1) : o;
+        if ((rc = run_phases(first_phase(), 1, o, direct))) return rc;
+        fused_cur = phase_set(2, o);
         FusedSlot<R>* fs = static_cast<FusedSlot<R>*>(slot_record);
         fs->ta = tick_args(fused_cur);
         fs->T = dT.p;
@@ -1159,9 +1242,21 @@ public:
 
     int fused_own_sweep() override {
         const bool direct = ovr_levels || ovr_eta_s || ovr_eta_t;
-        int rc = run_phase(2, fused_cur, direct);
+        int rc = run_phases(2, 2, cs, direct);
         if (rc) return rc;
         fused_own = true;
+        return MDL_OK;
+    }
+
+    int fused_whole() override {
+        if (inflight && (ovr_levels || ovr_eta_s || ovr_eta_t)) {
+            err = "fused_whole: replayed inputs apply to one barrier per completion";
+            return MDL_E_STATE;
+        }
+        if (!inflight) inflight_start = nbar;
+        int rc = run_barrier();
+        if (rc) return rc;
+        inflight += 1;
         return MDL_OK;
     }
 
@@ -1169,7 +1264,7 @@ public:
         const bool direct = ovr_levels || ovr_eta_s || ovr_eta_t;
         // the cooperative sweep runs the epilogue itself
         if (!(fused_own && coop_sweep)) {
-            int rc = run_phase(3, fused_cur, direct);
+            int rc = run_phases(3, 3, cs, direct);
             if (rc) return rc;
         }
         cs = fused_cur;

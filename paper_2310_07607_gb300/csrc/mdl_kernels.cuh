@@ -41,7 +41,7 @@ struct DevMeta {
     unsigned int changed;    // the adaptation changed the mesh
     unsigned int nf_pending; // non-finite values seen by this barrier's epilogue
     unsigned int cur_set;    // index of the state set holding the current values
-    unsigned int done_blocks;// epilogue blocks finished (last-block reduction)
+    unsigned int done_blocks;// blocks arrived at a kernel's last-block pass (0 between kernels)
     unsigned int cnt[8];     // elements per level b in this barrier
     int32_t nact[128];       // due elements per tick
     int64_t elem_updates;    // accumulated element steps
@@ -49,6 +49,7 @@ struct DevMeta {
     int64_t fac_updates;     // curved meshes: elements whose factors were computed
     double integral;         // FP64 int V after the last barrier
     unsigned int nfac;       // curved meshes: elements whose factors the adaptation recomputes
+    unsigned int adapted;    // this barrier's new mesh is committed and its state not yet transferred
     unsigned int gbar;       // cooperative sweep: arrivals at its grid barriers (zeroed before each launch)
 };
 
@@ -1089,16 +1090,50 @@ __global__ void __launch_bounds__(256, 1) k_tick(
     }
 }
 
+// Refinement marks of an adapting barrier, set by the kernel that computes the indicator: a leaf
+// whose eta^s reaches tau is marked unless it is at full depth, and under the 2:1 closure a marked
+// leaf marks its coarser face neighbours, theirs in turn, and so on.  Chains only go coarser, from a
+// leaf below full depth: up to max_refine - 1 leaves.  Two are followed here (a stack for longer ones
+// would give the kernel local memory, which cost 5 us a launch); k_amr_close takes the rest, a pass
+// per step.  The marks r are 0 at the start of the kernel (the level pass of the previous barrier
+// clears them); two threads that mark a leaf at once write the same.
+constexpr int MARK_CHAIN = 2;
+struct MarkArgs {
+    uint8_t* r;          // null: no adaptation
+    double tau;
+    int L;
+};
+
+template <int DIM>
+__device__ __forceinline__ void mark_leaf(const MarkArgs& a, const uint32_t* info, const int32_t* nbr, int64_t e,
+                                          uint32_t inf, double eta) {
+    constexpr int NF = 2 * DIM;
+    if (!(eta >= a.tau) || (int)((inf >> 24) & 15) >= a.L) return;
+    a.r[e] = 1;
+#pragma unroll 1
+    for (int f = 0; f < NF; ++f) {
+        if (((inf >> (4 * f)) & 3u) != 2u) continue;
+        const int32_t c = nbr[(size_t)e * NF + f];
+        const uint32_t ic = info[c];
+        a.r[c] = 1;
+#pragma unroll 1
+        for (int g = 0; g < NF; ++g)
+            if (((ic >> (4 * g)) & 3u) == 2u) a.r[nbr[(size_t)c * NF + g]] = 1;
+    }
+}
+
 // Kelly-type spatial indicator per element (Eq. dg-error-estimate) on the barrier-start
 // values; same-level and coarser neighbours are gathered before the face arithmetic.  In
 // FP32 the face-point sums are FP32 and the faces accumulate in FP64 (FP64 arithmetic per
-// face point would bound the kernel by the FP64 pipe).
+// face point would bound the kernel by the FP64 pipe).  Q1; see k_eta_s_q2 and k_eta_q23 for Q2.
 template <typename R, int DIM, int P>
-__global__ void k_eta_s(const DevArrays<R> d, const Tables<R> T, const Phys<R> ph) {
+__global__ void k_eta_s(const DevArrays<R> d, const Tables<R> T, const Phys<R> ph, const MarkArgs mark) {
+    static_assert(P == 1, "Q1");
     pdl_enter();
     using S = Shape<DIM, P>;
     constexpr int NP = S::NP, NF = S::NF, NSUB = S::NSUB, NPS = S::NPS;
     if (d.meta->err) return;
+    if (gtid() == 0) d.meta->changed = 0u;
     const int64_t ne = d.meta->ne;
     for (int64_t e = gtid(); e < ne; e += gstride()) {
         const uint32_t inf = d.info[e];
@@ -1146,31 +1181,6 @@ __global__ void k_eta_s(const DevArrays<R> d, const Tables<R> T, const Phys<R> p
                 for (int t = 0; t < NT; ++t) fsum += j[t] * j[t];
                 acc += (double)fsum;
             }
-        } else {
-            // Q2: the axis unrolled, the side a loop (half the code of a fully unrolled face
-            // loop; the kernel's size bounded it by instruction fetch)
-#pragma unroll
-            for (int k = 0; k < DIM; ++k)
-#pragma unroll 1
-            for (int side = 0; side < 2; ++side) {
-                const int f = 2 * k + side;
-                const int kind = (inf >> (4 * f)) & 3;
-                if (kind != 1 && kind != 2) continue;
-                const int s = side ? 1 : -1;
-                const int nbi = d.nbr[(size_t)e * NF + f];
-                const int pn = (d.lvl[nbi] >> 3) & 1;
-                const R* src = (pn ? d.V1 : d.V0) + (size_t)nbi * NPS;
-                R un[NP];
-                ld_dofs<R, NP, NPS>(src, un);
-                const int pos = (inf >> (4 * f + 2)) & 3;
-                if constexpr (sizeof(R) == 4)
-                    acc += ph.kfac[lev][k] * (double)face_kelly_sum<R, DIM, P>(T, ph, k, s, lev, -1, u,
-                                                                             kind == 1 ? lev : lev - 1,
-                                                                             kind == 1 ? -1 : pos, un, lev);
-                else
-                    acc += face_kelly<R, DIM, P>(T, ph, k, s, lev, -1, u, kind == 1 ? lev : lev - 1,
-                                                 kind == 1 ? -1 : pos, un, lev);
-            }
         }
         if constexpr (P == 1) {
 #pragma unroll
@@ -1196,79 +1206,269 @@ __global__ void k_eta_s(const DevArrays<R> d, const Tables<R> T, const Phys<R> p
                     acc += (double)fsum;
                 }
             }
-        } else {
-#pragma unroll
-            for (int k = 0; k < DIM; ++k)
-#pragma unroll 1
-            for (int side = 0; side < 2; ++side) {
-                const int f = 2 * k + side;
-                const int kind = (inf >> (4 * f)) & 3;
-                if (kind != 3) continue;
-                const int s = side ? 1 : -1;
-                const int h0 = d.nbr[(size_t)e * NF + f];
-                for (int sb = 0; sb < NSUB; ++sb) {
-                    const int nb = d.hang[h0 + sb];
-                    const int pn = (d.lvl[nb] >> 3) & 1;
-                    const R* src = (pn ? d.V1 : d.V0) + (size_t)nb * NPS;
-                    R un[NP];
-                    ld_dofs<R, NP, NPS>(src, un);
-                    if constexpr (sizeof(R) == 4)
-                        acc += ph.kfac[lev + 1][k] *
-                               (double)face_kelly_sum<R, DIM, P>(T, ph, k, s, lev, sb, u, lev + 1, -1, un, lev + 1);
-                    else
-                        acc += face_kelly<R, DIM, P>(T, ph, k, s, lev, sb, u, lev + 1, -1, un, lev + 1);
-                }
-            }
         }
-        d.eta_s[e] = sqrt(acc);
+        const double eta = sqrt(acc);
+        d.eta_s[e] = eta;
+        if (mark.r) mark_leaf<DIM>(mark, d.info, d.nbr, e, inf, eta);
     }
 }
 
+// Kelly term of one (sub)face of a Q2 element, sum_t w_t jump_t^2 (times the face weight of the
+// finer side's level, 4^lo and kfac): the flux jump at the face points from the traces of both
+// sides, one-dimensional derivatives along the face and, across a change of level, the
+// interpolation to the finer side's points.  to, dno: own trace and normal derivative; v: the
+// neighbour's values; kind 3: of subface pos.
+template <typename R, int DIM>
+__device__ __forceinline__ R kelly_face(const BoxOp<R>& op, const Tables<R>& T, int k, int side, int kind, int pos,
+                                        const R* to, const R* dno, const R* v) {
+    constexpr int NT = Shape<DIM, 2>::NT;
+    R tn[NT], dn[NT], dt[NT], dd[NT];
+    box_trace<R, DIM, 2>(op, k, 1 - side, v, tn, dn);
+    R ft = R(1);                       // tangential derivatives in the finer side's length
+    if (kind == 1) {
+#pragma unroll
+        for (int t = 0; t < NT; ++t) {
+            dd[t] = dno[t] - dn[t];
+            dt[t] = to[t] - tn[t];
+        }
+    } else {
+        // the coarser side's values at the finer side's points
+        R a[NT], b[NT];
+        const int c0 = pos & 1, c1 = (pos >> 1) & 1;
+        if (kind == 2) {
+            face_map<R, DIM, 2>(op.PR[0], c0, c1, tn, a);
+            face_map<R, DIM, 2>(op.PR[0], c0, c1, dn, b);
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {
+                dd[t] = dno[t] - R(0.5) * b[t];
+                dt[t] = to[t] - a[t];
+            }
+        } else {
+            face_map<R, DIM, 2>(op.PR[0], c0, c1, to, a);
+            face_map<R, DIM, 2>(op.PR[0], c0, c1, dno, b);
+            ft = R(2);
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {
+                dd[t] = b[t] - R(2) * dn[t];
+                dt[t] = a[t] - tn[t];
+            }
+        }
+    }
+    R j[NT];
+#pragma unroll
+    for (int t = 0; t < NT; ++t) j[t] = op.FK[k][k] * dd[t];
+    if (op.cross) {
+        int tg[2] = {0, 0};
+        tangents<DIM>(k, tg);
+#pragma unroll
+        for (int ti = 0; ti < DIM - 1; ++ti) face_line<R, DIM, 2>(op.D1, ti, ft * op.FK[k][tg[ti]], dt, j, true);
+    }
+    R s = R(0);
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+        const R w = DIM == 3 ? T.w[t % 3] * T.w[t / 3] : T.w[t];
+        s += w * j[t] * j[t];
+    }
+    return s;
+}
+
+// The indicator's terms of the two axis-K faces of a Q2 element from its values y; row(n, v): values of element n, both shifted
+// by a value of the element (the flux jump does not see a constant).  nbv(k, side, v): those of the
+// same-level neighbour of a face.
+template <typename R, int DIM, int K, typename ROW, typename NBV>
+__device__ __forceinline__ double kelly_axis(const DevArrays<R>& d, const BoxOp<R>& op, const Tables<R>& T,
+                                             const Phys<R>& ph, int64_t e, uint32_t inf, int lev, const R* y, ROW row,
+                                             NBV nbv) {
+    using S = Shape<DIM, 2>;
+    constexpr int NP = S::NP, NF = S::NF, NT = S::NT;
+    constexpr int k = K;
+    double acc = 0.0;
+    const R sc = R(1 << (2 * lev));
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side) {
+            const uint32_t fi = inf >> (8 * k + 4 * side);
+            const int kind = fi & 3;
+            if (kind == 0) continue;
+            R to[NT], dno[NT], v[NP];
+            box_trace<R, DIM, 2>(op, k, side, y, to, dno);
+            const int sb0 = kind == 3 ? 0 : (fi >> 2) & 3, sb1 = kind == 3 ? S::NSUB : sb0 + 1;
+            const int lf = kind == 3 ? lev + 1 : lev;
+            R s = R(0);
+#pragma unroll 1
+            for (int sb = sb0; sb < sb1; ++sb) {
+                if (kind == 1) nbv(k, side, v);
+                else {
+                    const int nbi = d.nbr[(size_t)e * NF + 2 * k + side];
+                    row(kind == 2 ? nbi : d.hang[nbi + sb], v);
+                }
+                s += kelly_face<R, DIM>(op, T, k, side, kind, sb, to, dno, v);
+            }
+            acc += ph.kfac[lf][k] * (double)(ph.Wface[lf][k] * sc * s);
+        }
+    return acc;
+}
+
+template <typename R, int DIM>
+__global__ void __launch_bounds__(128) k_eta_s_q2(const DevArrays<R> d, const Tables<R> T, const Phys<R> ph,
+                                                  const BoxOp<R> op, const MarkArgs mark) {
+    pdl_enter();
+    using S = Shape<DIM, 2>;
+    constexpr int NP = S::NP, NPS = S::NPS, NF = S::NF;
+    if (d.meta->err) return;
+    if (gtid() == 0) d.meta->changed = 0u;
+    const int64_t ne = d.meta->ne;
+    for (int64_t e = gtid(); e < ne; e += gstride()) {
+        const uint32_t inf = d.info[e];
+        R y[NP];
+        ld_dofs<R, NP, NPS>((((d.lvl[e] >> 3) & 1) ? d.V1 : d.V0) + (size_t)e * NPS, y);
+        const R c = y[NP / 2];
+        auto row = [&](int n, R* v) {
+            ld_dofs<R, NP, NPS>((((d.lvl[n] >> 3) & 1) ? d.V1 : d.V0) + (size_t)n * NPS, v);
+#pragma unroll
+            for (int q = 0; q < NP; ++q) v[q] -= c;
+        };
+#pragma unroll
+        for (int q = 0; q < NP; ++q) y[q] -= c;
+        auto nbv = [&](int k, int side, R* v) { row(d.nbr[(size_t)e * NF + 2 * k + side], v); };
+        const int lev = (inf >> 24) & 15;
+        double acc = kelly_axis<R, DIM, 0>(d, op, T, ph, e, inf, lev, y, row, nbv);
+        acc += kelly_axis<R, DIM, 1>(d, op, T, ph, e, inf, lev, y, row, nbv);
+        if constexpr (DIM == 3) acc += kelly_axis<R, DIM, DIM - 1>(d, op, T, ph, e, inf, lev, y, row, nbv);
+        const double eta = sqrt(acc);
+        d.eta_s[e] = eta;
+        if (mark.r) mark_leaf<DIM>(mark, d.info, d.nbr, e, inf, eta);
+    }
+}
+
+// Square root of a >= 0 in FP64 from an FP32 seed and two Newton steps (each squares the relative
+// error, 2^-22 to start with): 5 FP64 operations, which issue at 1/64 of the FP32 rate here.
+__device__ __forceinline__ double sqrt_seeded(double a) {
+    if (a == 0.0) return 0.0;
+    const float f = (float)a;
+    if (!(f > 1e-30f && f < 1e30f)) return sqrt(a);
+    const double y = (double)rsqrtf(f), h = 0.5 * y;
+    double s = a * y;
+    s = fma(fma(-s, s, a), h, s);
+    return fma(fma(-s, s, a), h, s);
+}
+
+// Sum as an unevaluated pair of FP32 values: s + c with |c| at most an ulp of s, 48 bits together.
+struct Pair {
+    float s, c;
+    // += w x, w = wh + wl
+    __device__ __forceinline__ void add(float wh, float wl, float x) {
+        const float p = wh * x;
+        const float e = fmaf(wl, x, fmaf(wh, x, -p));       // the product's rounding and the weight's tail
+        const float t = s + p, z = t - s;
+        c += ((s - (t - z)) + (p - z)) + e;                 // the sum's rounding
+        s = t;
+    }
+};
+
+// Weights of int V on box elements: GL weight products as pairs (0 past the last node) and the
+// level-0 volume factor; level l scales by 2^(-d l), exact.
+struct EpiWeights {
+    float wh[28], wl[28];
+    double w0;
+};
+
+__device__ __forceinline__ double warp_sum(double x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+// Sum over the block (of at most 1024 threads), valid in thread 0.
+__device__ __forceinline__ double block_sum(double x) {
+    __shared__ double part[32];
+    x = warp_sum(x);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = x;
+    __syncthreads();
+    if (threadIdx.x < 32) x = warp_sum(threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0.0);
+    __syncthreads();
+    return x;
+}
+
 // Barrier epilogue: eta^t = sqrt(acc)/dt, parity flip of single-step elements, non-finite
-// check, per-block partial sums of int V = sum_q M_q V_q (FP64).
+// check, per-block partial sums of int V = sum_q M_q V_q.  FP64 sums bound it (1.25 TFLOP/s: 0.3 ms
+// for 2.6M Q2 elements, two FP64 instructions a DOF), so FP32 contexts on box elements sum pairs of
+// FP32 values with the FP64 precision's weights; the threads' sums are FP64.  Rows of 27 values are
+// read by whole warps (see mdl_q23.cuh), shorter ones by their element's thread.
 template <typename R, int DIM, int P>
 __global__ void __launch_bounds__(256) k_epilogue(const DevArrays<R> d, const double* __restrict__ mtab,
-                                                 double dt, double inv_dt, int inv_dt_exact, int mass_per_elem) {
+                                                 const EpiWeights ew, double dt, double inv_dt, int inv_dt_exact,
+                                                 int mass_per_elem) {
     pdl_enter();
     using S = Shape<DIM, P>;
-    constexpr int NP = S::NP;
-    __shared__ double red[256];
+    constexpr int NP = S::NP, NPS = S::NPS;
+    constexpr bool PAIRS = sizeof(R) == 4, COOP = PAIRS && NPS != NP;
     if (d.meta->err) return;
     const int64_t ne = d.meta->ne;
     double loc = 0.0;
-    bool bad = false;
-    for (int64_t e = gtid(); e < ne; e += gstride()) {
-        // eta^t = sqrt(acc) / dt in FP64 (it sets b^cell); the product with 1/dt equals the
-        // quotient whenever dt is a power of two, as the automatic barrier step is
-        d.eta_t[e] = inv_dt_exact ? sqrt(d.acc[e]) * inv_dt : sqrt(d.acc[e]) / dt;
-        uint8_t lv = d.lvl[e];
-        if ((lv & 7) == 0) {
-            lv ^= 8;
-            d.lvl[e] = lv;
+    Pair sum{0.0f, 0.0f};
+    float nf = 0.0f;                 // not 0 once a value was not finite
+    const int lane = threadIdx.x & 31;
+    for (int64_t base = gtid() - lane; base < ne; base += gstride()) {
+        const int64_t e = base + lane;
+        const bool in = e < ne;
+        uint8_t lv = 0;
+        int lev = 0;
+        if (in) {
+            // eta^t = sqrt(acc) / dt in FP64 (it sets b^cell); the product with 1/dt equals the
+            // quotient whenever dt is a power of two, as the automatic barrier step is
+            const double a = d.acc[e], r = PAIRS ? sqrt_seeded(a) : sqrt(a);
+            d.eta_t[e] = inv_dt_exact ? r * inv_dt : r / dt;
+            lv = d.lvl[e];
+            if ((lv & 7) == 0) {
+                lv ^= 8;
+                d.lvl[e] = lv;
+            }
+            lev = (d.info[e] >> 24) & 15;
         }
-        const int par = (lv >> 3) & 1;
-        const R* Vc = (par ? d.V1 : d.V0) + (size_t)e * S::NPS;
-        const R* w = d.v + (size_t)e * S::NPS;
-        const int lev = (d.info[e] >> 24) & 15;
-        // GL masses: per (level, node) on box elements, per (element, node) on mapped ones
-        const double* Mq = mtab + (mass_per_elem ? (size_t)e * NP : (size_t)lev * NP);
+        const R* Vc = (((lv >> 3) & 1) ? d.V1 : d.V0) + (size_t)(in ? e : base) * NPS;
+        const R* w = d.v + (size_t)(in ? e : base) * NPS;
+        if (COOP && !mass_per_elem) {
+            if constexpr (COOP) {
+                const float sl = in ? pow2_neg<float>(DIM * lev) : 0.0f;
 #pragma unroll
-        for (int q = 0; q < NP; ++q) {
-            const R x = Vc[q];
-            loc += Mq[q] * (double)x;
-            bad = bad || !isfinite(x) || !isfinite(w[q]);
+                for (int j = 0; j < 7; ++j) {
+                    const int t = 32 * j + lane, r = t / 7, c = t - 7 * r;
+                    const float4 x = reinterpret_cast<const float4*>(__shfl_sync(0xffffffffu, (long long)Vc, r))[c];
+                    const float4 y = reinterpret_cast<const float4*>(__shfl_sync(0xffffffffu, (long long)w, r))[c];
+                    const float sr = __shfl_sync(0xffffffffu, sl, r);
+                    sum.add(ew.wh[4 * c], ew.wl[4 * c], sr * x.x);
+                    sum.add(ew.wh[4 * c + 1], ew.wl[4 * c + 1], sr * x.y);
+                    sum.add(ew.wh[4 * c + 2], ew.wl[4 * c + 2], sr * x.z);
+                    sum.add(ew.wh[4 * c + 3], ew.wl[4 * c + 3], sr * x.w);
+                    nf += 0.0f * x.x + 0.0f * x.y + 0.0f * x.z + 0.0f * x.w;
+                    nf += 0.0f * y.x + 0.0f * y.y + 0.0f * y.z + 0.0f * y.w;
+                }
+            }
+        } else if (in) {
+            R x[NP], y[NP];
+            ld_dofs<R, NP, NPS>(Vc, x);
+            ld_dofs<R, NP, NPS>(w, y);
+            if (PAIRS && !mass_per_elem) {
+                const float sl = pow2_neg<float>(DIM * lev);
+#pragma unroll
+                for (int q = 0; q < NP; ++q) sum.add(ew.wh[q], ew.wl[q], sl * (float)x[q]);
+            } else {
+                // GL masses: per (level, node) on box elements, per (element, node) on mapped ones
+                const double* Mq = mtab + (mass_per_elem ? (size_t)e * NP : (size_t)lev * NP);
+#pragma unroll
+                for (int q = 0; q < NP; ++q) loc += Mq[q] * (double)x[q];
+            }
+#pragma unroll
+            for (int q = 0; q < NP; ++q)
+                if (!isfinite(x[q]) || !isfinite(y[q])) nf = 1.0f;
         }
     }
-    if (bad) atomicOr(&d.meta->nf_pending, 1u);
-    red[threadIdx.x] = loc;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
-    }
+    if (PAIRS && !mass_per_elem) loc = ((double)sum.s + (double)sum.c) * ew.w0;
+    if (!(nf == 0.0f)) atomicOr(&d.meta->nf_pending, 1u);
+    loc = block_sum(loc);
     __shared__ bool last;
     if (threadIdx.x == 0) {
-        d.partial[blockIdx.x] = red[0];
+        d.partial[blockIdx.x] = loc;
         __threadfence();
         last = atomicAdd(&d.meta->done_blocks, 1u) == gridDim.x - 1;
     }
@@ -1277,19 +1477,14 @@ __global__ void __launch_bounds__(256) k_epilogue(const DevArrays<R> d, const do
     // the last block: fixed-order sum of the partials, barrier count, non-finite flag
     __threadfence();
     double s2 = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) s2 += ((volatile double*)d.partial)[i];
-    red[threadIdx.x] = s2;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
-    }
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) s2 += __ldcg(d.partial + i);
+    s2 = block_sum(s2);
     if (threadIdx.x == 0) {
         DevMeta* m = d.meta;
-        m->integral = red[0];
+        m->integral = s2;
         m->nbar += 1;
         m->done_blocks = 0;
-        if (m->nf_pending) {
+        if (*(volatile unsigned*)&m->nf_pending) {
             m->err |= ERR_NONFINITE;
             m->nf_pending = 0;
         }
@@ -1719,158 +1914,6 @@ __global__ void k_lat_refresh(DevArrays<R> d, const Tables<R> T, const Phys<R> p
     }
     inf = pending ? (inf | INFO_PENDING) : (inf & ~INFO_PENDING);
     d.info[e] = inf;
-    }
-}
-
-// Solution transfer after adaptation (Alg. 1 adapt steps): keep, prolong (parent
-// polynomial at the child nodes) or restrict (L2 projection with the children's GL
-// rule, exact for the diagonal GL mass).  Old arrays in `o`, new in `n` (slot 0).  Kept
-// elements (most of them) with rows of 27 values are copied by whole warps: a warp takes 32
-// consecutive new elements and copies their rows lane-parallel over the values, the old row
-// of each element broadcast from its lane; shorter rows, refined and coarsened elements take
-// a thread each.
-template <typename R, int DIM, int P>
-__global__ void k_transfer(const DevArrays<R> o, DevArrays<R> n, const int8_t* pkind, const int32_t* psrc,
-                           const int8_t* pbits, const Tables<R> T) {
-    pdl_enter();
-    using S = Shape<DIM, P>;
-    constexpr int N1 = S::N1, NP = S::NP, NC = 1 << DIM, NPS = S::NPS;
-    if (n.meta->err) return;
-    const int64_t nne = n.meta->ne;
-    if constexpr (NP < 27) {
-        // short rows (Q1, 2D Q2): a thread per kept element
-        for (int64_t i = gtid(); i < nne; i += gstride()) {
-            if (pkind[i] != 0) continue;
-            const int src = psrc[i];
-            const int par = (o.lvl[src] >> 3) & 1;
-            const R* Vo = (par ? o.V1 : o.V0) + (size_t)src * NPS;
-            const R* wo = o.v + (size_t)src * NPS;
-#pragma unroll
-            for (int q = 0; q < NPS; ++q) {
-                n.V0[(size_t)i * NPS + q] = Vo[q];
-                n.v[(size_t)i * NPS + q] = wo[q];
-            }
-            n.eta_t[i] = o.eta_t[src];
-            n.lvl[i] = 0;
-        }
-    } else {
-        const int lane = threadIdx.x & 31;
-        const int64_t nwarp = gstride() >> 5;
-        for (int64_t base = (gtid() >> 5) * 32; base < nne; base += nwarp * 32) {
-            const int64_t i = base + lane;
-            long long vrow = 0, wrow = 0;   // old rows of a kept element (0: not kept)
-            if (i < nne && pkind[i] == 0) {
-                const int src = psrc[i];
-                const int par = (o.lvl[src] >> 3) & 1;
-                vrow = (long long)((par ? o.V1 : o.V0) + (size_t)src * NPS);
-                wrow = (long long)(o.v + (size_t)src * NPS);
-                n.eta_t[i] = o.eta_t[src];
-                n.lvl[i] = 0;
-            }
-            // value idx = lane + 32 j of the warp's block of padded rows: row r = idx / NPS,
-            // column q (the pad copied too); every load of the block is issued before the
-            // first store
-            R xv[NPS], xw[NPS];
-            bool keep[NPS];
-            int r = lane / NPS, q = lane - (lane / NPS) * NPS;
-#pragma unroll
-            for (int j = 0; j < NPS; ++j) {
-                const long long vr = __shfl_sync(0xffffffffu, vrow, r);
-                const long long wr = __shfl_sync(0xffffffffu, wrow, r);
-                keep[j] = vr != 0;
-                xv[j] = keep[j] ? reinterpret_cast<const R*>(vr)[q] : R(0);
-                xw[j] = keep[j] ? reinterpret_cast<const R*>(wr)[q] : R(0);
-                q += 32 % NPS;
-                r += 32 / NPS;
-                if (q >= NPS) {
-                    q -= NPS;
-                    ++r;
-                }
-            }
-            const size_t o0 = (size_t)base * NPS + lane;
-#pragma unroll
-            for (int j = 0; j < NPS; ++j) {
-                if (keep[j]) {
-                    n.V0[o0 + 32 * j] = xv[j];
-                    n.v[o0 + 32 * j] = xw[j];
-                }
-            }
-        }
-    }
-    for (int64_t i = gtid(); i < nne; i += gstride()) {
-    const int kd = pkind[i];
-    if (kd == 0) continue;
-    const int src = psrc[i];
-    R* Vn = n.V0 + (size_t)i * NPS;
-    R* wn = n.v + (size_t)i * NPS;
-#pragma unroll
-    for (int q = NP; q < NPS; ++q) Vn[q] = wn[q] = R(0);
-    if (kd == 1) {
-        const int bits = pbits[i];
-        const int par = (o.lvl[src] >> 3) & 1;
-        const R* Vo = (par ? o.V1 : o.V0) + (size_t)src * NPS;
-        const R* wo = o.v + (size_t)src * NPS;
-#pragma unroll
-        for (int q = 0; q < NP; ++q) {
-            R a = 0, c = 0;
-            for (int j = 0; j < NP; ++j) {
-                R w = R(1);
-#pragma unroll
-                for (int k = 0; k < DIM; ++k) w *= T.Pi[(bits >> k) & 1][digit<N1>(q, k)][digit<N1>(j, k)];
-                a += w * Vo[j];
-                c += w * wo[j];
-            }
-            Vn[q] = a;
-            wn[q] = c;
-        }
-        n.eta_t[i] = o.eta_t[src];
-    } else {
-        R a[NP], c[NP];
-#pragma unroll
-        for (int q = 0; q < NP; ++q) a[q] = c[q] = R(0);
-        double et = 0.0;
-        for (int cb = 0; cb < NC; ++cb) {
-            const int ch = src + cb;
-            const int par = (o.lvl[ch] >> 3) & 1;
-            const R* Vo = (par ? o.V1 : o.V0) + (size_t)ch * NPS;
-            const R* wo = o.v + (size_t)ch * NPS;
-            et += o.eta_t[ch];
-            for (int qc = 0; qc < NP; ++qc) {
-                // the child's GL weight in the parent's measure; on a mapped mesh the child's
-                // own GL mass (divided by the parent's below)
-                R wc = R(1);
-                if (o.mq) {
-                    wc = (R)o.mq[(size_t)ch * NP + qc];
-                } else {
-#pragma unroll
-                    for (int k = 0; k < DIM; ++k) wc *= T.w[digit<N1>(qc, k)] * R(0.5);
-                }
-                const R xv = wc * Vo[qc], xw = wc * wo[qc];
-#pragma unroll
-                for (int q = 0; q < NP; ++q) {
-                    R w = R(1);
-#pragma unroll
-                    for (int k = 0; k < DIM; ++k) w *= T.Pi[(cb >> k) & 1][digit<N1>(qc, k)][digit<N1>(q, k)];
-                    a[q] += w * xv;
-                    c[q] += w * xw;
-                }
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < NP; ++q) {
-            R wq = R(1);
-            if (n.mq) {
-                wq = (R)n.mq[(size_t)i * NP + q];
-            } else {
-#pragma unroll
-                for (int k = 0; k < DIM; ++k) wq *= T.w[digit<N1>(q, k)];
-            }
-            Vn[q] = a[q] / wq;
-            wn[q] = c[q] / wq;
-        }
-        n.eta_t[i] = et / NC;
-    }
-    n.lvl[i] = 0;
     }
 }
 

@@ -373,12 +373,14 @@ __device__ __forceinline__ void tick_elem_mapped(const TickArgs<R>& a, const Tab
 // W_F(t) = dS_t / (reference GL weight of t): h_F / (2p) sum_t dS_t (W_F(t) J_t)^2.  Face-point
 // sums in the working precision, faces accumulated in FP64.
 template <typename R, int DIM, int P>
-__global__ void __launch_bounds__(128) k_eta_s_mapped(const DevArrays<R> d, const Tables<R> T) {
+__global__ void __launch_bounds__(128) k_eta_s_mapped(const DevArrays<R> d, const Tables<R> T,
+                                                       const MarkArgs mark) {
     pdl_enter();
     using M = MapShape<DIM, P>;
     constexpr int N1 = M::N1, NP = M::NP, NF = M::NF, NPF = M::NPF, FPV = M::FPV;
     constexpr int NPS = Shape<DIM, P>::NPS;
     if (d.meta->err) return;
+    if (gtid() == 0) d.meta->changed = 0u;
     const int64_t ne = d.meta->ne;
     for (int64_t e = gtid(); e < ne; e += gstride()) {
         const uint32_t inf = d.info[e];
@@ -450,7 +452,9 @@ __global__ void __launch_bounds__(128) k_eta_s_mapped(const DevArrays<R> d, cons
             }
             face_sum(dS, jmp);
         }
-        d.eta_s[e] = sqrt(acc);
+        const double eta = sqrt(acc);
+        d.eta_s[e] = eta;
+        if (mark.r) mark_leaf<DIM>(mark, d.info, d.nbr, e, inf, eta);
     }
 }
 

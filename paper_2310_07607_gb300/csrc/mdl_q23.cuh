@@ -23,6 +23,7 @@ constexpr int NP = 27, NPS = 28, NT = 9, NF = 6;
 constexpr int ROWS = 5;                                   // blocks of 32 rows: A0, A1, B0, B1, own values
 constexpr int BLK = 32 * NPS;                             // floats of a block
 constexpr int smem_bytes(int threads) { return ROWS * NPS * 4 * threads; }
+constexpr int eta_smem_bytes(int threads) { return 4 * NPS * 4 * threads; }
 
 // Row r of the warp's block dst from lane r's `row`: chunk t = 32 j + lane is chunk t % 7 of row
 // t / 7, and the block is contiguous.
@@ -96,7 +97,12 @@ __global__ void __launch_bounds__(384, 1) k_tick_q23(const TickArgs<float> a, co
     const int lane = threadIdx.x & 31;
     const int G = (int)gstride();
     int base = (int)gtid() - lane;                         // the warp's first due element
-    if (base >= n_act) return;
+    // a warp without an element leaves its SM to other work; a tick without any must still end after
+    // the tick before it (the next one waits for this one only)
+    if (base >= n_act) {
+        if (n_act == 0) pdl_enter();
+        return;
+    }
     // a warp's blocks of rows, and the thread's row in each
     float* const A0 = rows + (size_t)(threadIdx.x >> 5) * ROWS * BLK;
     float *const A1 = A0 + BLK, *const B0 = A0 + 2 * BLK, *const B1 = A0 + 3 * BLK, *const U = A0 + 4 * BLK;
@@ -284,6 +290,80 @@ __global__ void __launch_bounds__(384, 1) k_tick_q23(const TickArgs<float> a, co
         base += G;
         if (base >= n_act) return;
         __syncwarp();                                      // the blocks are read: the next rows may land
+    }
+}
+
+// The spatial indicator of Q2 3D FP32 contexts (k_eta_s_q2's sums) with the same row copies: the
+// own rows and axis 0, then two axes ahead in turn.
+template <int DIM, int P>
+__global__ void __launch_bounds__(128, 4) k_eta_q23(const DevArrays<float> d, const Tables<float> T,
+                                                   const Phys<float> ph, const BoxOp<float> op, const MarkArgs mark) {
+    static_assert(DIM == 3 && P == 2, "Q2 3D only");
+    using namespace q23;
+    extern __shared__ __align__(16) float rows[];
+    pdl_enter();
+    if (d.meta->err) return;
+    if (gtid() == 0) d.meta->changed = 0u;
+    const int64_t ne = d.meta->ne;
+    const int lane = threadIdx.x & 31;
+    float* const A0 = rows + (size_t)(threadIdx.x >> 5) * 4 * BLK;
+    const int my = lane * NPS;
+    for (int64_t base = gtid() - lane; base < ne; base += gstride()) {
+        const bool valid = base + lane < ne;
+        const int e = (int)(valid ? base + lane : ne - 1);
+        const uint32_t inf = d.info[e];
+        const int lev = (inf >> 24) & 15;
+        int nbf[NF];
+        uint8_t lvn[NF];
+#pragma unroll
+        for (int f = 0; f < NF; f += 2) {
+            const int2 x = *reinterpret_cast<const int2*>(d.nbr + (size_t)e * NF + f);
+            nbf[f] = ((inf >> (4 * f)) & 3) == 1 ? x.x : e;
+            nbf[f + 1] = ((inf >> (4 * f + 4)) & 3) == 1 ? x.y : e;
+        }
+        const uint8_t lv = d.lvl[e];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) lvn[f] = d.lvl[nbf[f]];
+        auto value_row = [&](int n, uint8_t l) { return (((l >> 3) & 1) ? d.V1 : d.V0) + (size_t)n * NPS; };
+        auto stage_axis = [&](int k, float* r0) {
+            copy_rows(r0, value_row(nbf[2 * k], lvn[2 * k]), lane);
+            copy_rows(r0 + BLK, value_row(nbf[2 * k + 1], lvn[2 * k + 1]), lane);
+            copy_commit();
+        };
+        __syncwarp();                                   // the blocks of the last elements are read
+        copy_rows(A0 + 2 * BLK, value_row(e, lv), lane);
+        stage_axis(0, A0);
+        copy_wait<0>();
+        float t[NPS], y[NP];
+        ld_vec<float, NPS>(A0 + 2 * BLK + my, t);
+        const float c = t[NP / 2];
+#pragma unroll
+        for (int q = 0; q < NP; ++q) y[q] = t[q] - c;
+        __syncwarp();
+        stage_axis(1, A0 + 2 * BLK);
+        auto row = [&](int n, float* v) {
+            ld_dofs<float, NP, NPS>(value_row(n, d.lvl[n]), v);
+#pragma unroll
+            for (int q = 0; q < NP; ++q) v[q] -= c;
+        };
+        auto nbv = [&](int k, int side, float* v) {
+            float x[NPS];
+            ld_vec<float, NPS>(A0 + (k == 1 ? 2 * BLK : 0) + side * BLK + my, x);
+#pragma unroll
+            for (int q = 0; q < NP; ++q) v[q] = x[q] - c;
+        };
+        double acc = kelly_axis<float, DIM, 0>(d, op, T, ph, e, inf, lev, y, row, nbv);
+        __syncwarp();
+        stage_axis(2, A0);
+        copy_wait<1>();
+        acc += kelly_axis<float, DIM, 1>(d, op, T, ph, e, inf, lev, y, row, nbv);
+        copy_wait<0>();
+        acc += kelly_axis<float, DIM, 2>(d, op, T, ph, e, inf, lev, y, row, nbv);
+        if (valid) {
+            const double eta = sqrt_seeded(acc);
+            d.eta_s[e] = eta;
+            if (mark.r) mark_leaf<DIM>(mark, d.info, d.nbr, e, inf, eta);
+        }
     }
 }
 

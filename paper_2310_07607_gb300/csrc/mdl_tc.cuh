@@ -285,7 +285,10 @@ __global__ void __launch_bounds__(tc::THREADS, 2)
     // tick skips the set-up and leaves its SM to other work (a small instance's fine ticks)
     const int n_act = d.meta->nact[tick];
     const int ntiles = (n_act + M - 1) / M;
-    if ((int)blockIdx.x >= ntiles) return;
+    if ((int)blockIdx.x >= ntiles) {
+        if (ntiles == 0) pdl_enter();   // the next tick waits for this one only, and this one for the last
+        return;
+    }
 
     // --- set-up that reads nothing the previous tick writes (before the dependent wait)
     // the operator's FP16 terms, stored in global memory as the image of their swizzled shared-
