@@ -251,6 +251,9 @@ class Ctx : public CtxBase {
     static constexpr int MAP_VOL = NP * (DIM * (DIM + 1) / 2 + 1);      // factor values per element
     static constexpr int MAP_FACE = NF * (DIM == 2 ? N1 : N1 * N1) * (DIM + 2);
 
+    // Elements with room for their factors: whole groups of 32.
+    static int64_t fac_elems(int64_t c) { return (c + 31) / 32 * 32; }
+
     int alloc_set(Set& x, int64_t c) {
         MDL_CK(x.V0.ensure((size_t)c * NPS));
         MDL_CK(x.V1.ensure((size_t)c * NPS));
@@ -259,8 +262,8 @@ class Ctx : public CtxBase {
         MDL_CK(x.lvl.ensure(c));
         MDL_CK(x.coord.ensure(c));
         if (mapped) {
-            MDL_CK(x.gvol.ensure((size_t)c * MAP_VOL));
-            MDL_CK(x.gface.ensure((size_t)c * MAP_FACE));
+            MDL_CK(x.gvol.ensure((size_t)fac_elems(c) * MAP_VOL));
+            MDL_CK(x.gface.ensure((size_t)fac_elems(c) * MAP_FACE));
             MDL_CK(x.mq.ensure((size_t)c * NP));
             MDL_CK(x.fsig.ensure(c));
             for (int s = 0; s < pb.n_stim; ++s) MDL_CK(x.fsm[s].ensure(c));
@@ -323,7 +326,9 @@ class Ctx : public CtxBase {
         MDL_GROW(x.V0, NPS); MDL_GROW(x.V1, NPS); MDL_GROW(x.v, NPS); MDL_GROW(x.eta_t, 1);
         MDL_GROW(x.lvl, 1); MDL_GROW(x.coord, 1);
         if (mapped) {
-            MDL_GROW(x.gvol, MAP_VOL); MDL_GROW(x.gface, MAP_FACE); MDL_GROW(x.mq, NP); MDL_GROW(x.fsig, 1);
+            if ((rc = grow_copy(x.gvol, (size_t)fac_elems(c) * MAP_VOL, (size_t)fac_elems(ne) * MAP_VOL))) return rc;
+            if ((rc = grow_copy(x.gface, (size_t)fac_elems(c) * MAP_FACE, (size_t)fac_elems(ne) * MAP_FACE))) return rc;
+            MDL_GROW(x.mq, NP); MDL_GROW(x.fsig, 1);
             for (int s = 0; s < pb.n_stim; ++s) MDL_GROW(x.fsm[s], 1);
         }
         MDL_GROW(bcfl, 1); MDL_GROW(info, 1); MDL_GROW(loc, 1); MDL_GROW(nbr, NF); MDL_GROW(hang, NF * NSUB);

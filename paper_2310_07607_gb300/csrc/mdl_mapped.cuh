@@ -1,6 +1,9 @@
 // mdl_mapped.cuh -- the element step on curved (mapped) meshes: thread per element.
 //
-// The geometric factors of every element (mdl_geometry.h) are stored per GL point: at volume
+// The geometric factors of every element (mdl_geometry.h) are stored per GL point, in groups of
+// 32 elements with the element fastest (value i of element e at [e / 32][i][e % 32]): a warp takes
+// consecutive elements, and a row of 704 bytes per element (Q1 3D) read value by value by its own
+// thread is 32 cache lines an instruction.  At volume
 // node q the symmetric metric G_q and the mass M_q, at face point t the flux vector c, the
 // area weight dS and the penalty kappa.  The residual of element e (Eq. monodomain-primal-
 // formulation with the flux of Eq. monodomain-numerical-flux, all faces conforming):
@@ -26,7 +29,15 @@ struct MapShape {
     static constexpr int NS = DIM * (DIM + 1) / 2;
     static constexpr int VPN = NS + 1;        // values per volume node: G, M
     static constexpr int FPV = DIM + 2;       // values per face point: c, dS, kappa
+    static constexpr int NV = NP * VPN, NFV = NF * NPF * FPV;   // factor values per element
 };
+
+// Factors of element e, `per` values each, FS apart.
+constexpr int FS = 32;
+template <typename R>
+__device__ __forceinline__ R* factors_of(R* base, int64_t e, int per) {
+    return base + (size_t)(e >> 5) * per * FS + (e & 31);
+}
 
 // Entry (k, l) of the symmetric metric stored as (xx, yy, xy) or (xx, yy, zz, xy, xz, yz).
 template <int DIM>
@@ -84,8 +95,8 @@ __device__ __forceinline__ void mapped_face_fluxes(const Tables<R>& T, const R* 
 #pragma unroll
     for (int t = 0; t < NPF; ++t) {
         const int at[2] = {t % N1, t / N1};
-        const R* c = gf + t * FPV;
-        R fo = c[k] * go[t], fn = c[k] * gn[t];
+        const R* c = gf + t * FPV * FS;
+        R fo = c[k * FS] * go[t], fn = c[k * FS] * gn[t];
 #pragma unroll
         for (int z = 0; z < DIM - 1; ++z) {
             const int st = z == 0 ? 1 : N1;            // face-point stride of tangent z
@@ -96,8 +107,8 @@ __device__ __forceinline__ void mapped_face_fluxes(const Tables<R>& T, const R* 
                 so += T.D1[at[z]][a] * to[t2];
                 sn += T.D1[at[z]][a] * tn[t2];
             }
-            fo += c[tg[z]] * so;
-            fn += c[tg[z]] * sn;
+            fo += c[tg[z] * FS] * so;
+            fn += c[tg[z] * FS] * sn;
         }
         flo[t] = fo;
         fln[t] = fn;
@@ -131,7 +142,7 @@ __device__ __forceinline__ void face_point_eval(const Tables<R>& T, const R* v, 
                 if (DIM == 3) g1 += bs[m] * L[0][m0] * DL[1][m1] * val;
             }
     tr = t;
-    fl = cscale * (c[k] * gn + c[tg[0]] * g0 + (DIM == 3 ? c[tg[1]] * g1 : R(0)));
+    fl = cscale * (c[k * FS] * gn + c[tg[0] * FS] * g0 + (DIM == 3 ? c[tg[1] * FS] * g1 : R(0)));
 }
 
 // r_i += A psi_i + Bc cscale c . grad_xi psi_i at such a point.
@@ -152,8 +163,8 @@ __device__ __forceinline__ void face_point_distribute(const Tables<R>& T, int k,
                 const int node = m * stride<N1>(k) + m0 * stride<N1>(tg[0]) + (DIM == 3 ? m1 * stride<N1>(tg[1]) : 0);
                 const R l1 = DIM == 3 ? L[1][m1] : R(1);
                 const R psi = bs[m] * L[0][m0] * l1;
-                const R cg = c[k] * ds[m] * L[0][m0] * l1 + c[tg[0]] * bs[m] * DL[0][m0] * l1 +
-                             (DIM == 3 ? c[tg[1]] * bs[m] * L[0][m0] * DL[1][m1] : R(0));
+                const R cg = c[k * FS] * ds[m] * L[0][m0] * l1 + c[tg[0] * FS] * bs[m] * DL[0][m0] * l1 +
+                             (DIM == 3 ? c[tg[1] * FS] * bs[m] * L[0][m0] * DL[1][m1] : R(0));
                 r[node] += A * psi + Bs * cg;
             }
 }
@@ -182,30 +193,31 @@ __device__ __forceinline__ void half_rows(const Tables<R>& T, int t, int bits, R
 // its own values on the half of its face the subface covers.
 template <typename R, int DIM, int P>
 __device__ __forceinline__ void mapped_hanging_coarse(const DevArrays<R>& d, const Tables<R>& T, int tick, int B,
-                                                      int e, int f, const R* u, R* r) {
+                                                      int e, int k, int sd, const R* u, R* r) {
     using M = MapShape<DIM, P>;
     constexpr int NP = M::NP, NF = M::NF, NPF = M::NPF, FPV = M::FPV, NSUB = 1 << (DIM - 1);
     constexpr int NPS = Shape<DIM, P>::NPS;
-    const int k = f >> 1, sd = f & 1;
+    const int f = 2 * k + sd;
     int tg[2] = {0, 0};
     face_tangents<DIM>(k, tg);
     const int base = d.nbr[(size_t)e * NF + f];
+#pragma unroll 1
     for (int sb = 0; sb < NSUB; ++sb) {
         const int j = d.hang[base + sb];
         R uj[NP];
         load_seen<R, NP, NPS>(d, tick, B, j, uj);
-        const R* gfj = d.gface + ((size_t)j * NF + (f ^ 1)) * NPF * FPV;
+        const R* gfj = factors_of(d.gface, j, M::NFV) + (f ^ 1) * NPF * FPV * FS;
         R tj[NPF], tx[NPF], fj[NPF], fx[NPF];
         mapped_face_fluxes<R, DIM, P>(T, uj, uj, k, sd ^ 1, gfj, tj, tx, fj, fx);
 #pragma unroll
         for (int t = 0; t < NPF; ++t) {
-            const R* c = gfj + t * FPV;
+            const R* c = gfj + t * FPV * FS;
             R L[2][P + 1], DL[2][P + 1];
             half_rows<R, DIM, P>(T, t, sb, L, DL);
             R tro, flo;
             face_point_eval<R, DIM, P>(T, u, k, sd, tg, L, DL, c, R(-0.5), tro, flo);
             const R fln = -fj[t];
-            const R dS = c[DIM], kap = c[DIM + 1];
+            const R dS = c[DIM * FS], kap = c[(DIM + 1) * FS];
             const R jump = tro - tj[t];
             const R A = dS * (R(-0.5) * (flo + fln) + kap * jump);
             const R Bc = R(-0.5) * dS * jump;
@@ -215,16 +227,35 @@ __device__ __forceinline__ void mapped_hanging_coarse(const DevArrays<R>& d, con
 }
 
 template <typename R, int DIM, int P>
-__device__ __forceinline__ void mapped_residual(const DevArrays<R>& d, const Tables<R>& T, int tick, int B, int e,
-                                                uint32_t inf, const R* u, R* r) {
+__device__ __forceinline__ void mapped_residual(const DevArrays<R>& d, const Tables<R>& T, int tick, int B,
+                                                const TickMeta<DIM, P>& mt, const R* u, R* r) {
     using M = MapShape<DIM, P>;
     constexpr int N1 = M::N1, NP = M::NP, NF = M::NF, NPF = M::NPF, VPN = M::VPN, FPV = M::FPV;
     constexpr int NPS = Shape<DIM, P>::NPS;
+    const int e = mt.e;
+    const uint32_t inf = mt.inf;
+    // the neighbours' rows: FP32 Q1 all at once (48 registers), else face by face
+    constexpr bool ALL = sizeof(R) == 4 && P == 1;
+    R un_[ALL ? NF : 1][NP];
+    if constexpr (ALL) {
+        const R* ol[NF];
+        R th[NF];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            const int kind = (inf >> (4 * f)) & 3;
+            const bool use = kind == 1 || kind == 2;
+            ld_dofs<R, NP, NPS>(
+                seen_row<R, NPS>(d, tick, B, use ? mt.nbf[f] : e, use ? mt.lvn[f] : mt.lv, ol[f], th[f]), un_[f]);
+        }
+#pragma unroll
+        for (int f = 0; f < NF; ++f)
+            if (th[f] > R(0)) interp_row<R, NP, NPS>(ol[f], th[f], un_[f]);
+    }
 #pragma unroll
     for (int q = 0; q < NP; ++q) r[q] = R(0);
     // volume: flux G_q grad u at every node, then r_i = sum_k sum_m D1[m][a_k(i)] flux_k(node m of i's line)
     {
-        const R* gv = d.gvol + (size_t)e * NP * VPN;
+        const R* gv = factors_of(d.gvol, e, M::NV);
         R fl[NP][DIM];
 #pragma unroll
         for (int q = 0; q < NP; ++q) {
@@ -241,7 +272,7 @@ __device__ __forceinline__ void mapped_residual(const DevArrays<R>& d, const Tab
             for (int k = 0; k < DIM; ++k) {
                 R s = R(0);
 #pragma unroll
-                for (int l = 0; l < DIM; ++l) s += gv[q * VPN + sym_index<DIM>(k, l)] * g[l];
+                for (int l = 0; l < DIM; ++l) s += gv[(q * VPN + sym_index<DIM>(k, l)) * FS] * g[l];
                 fl[q][k] = s;
             }
         }
@@ -257,24 +288,24 @@ __device__ __forceinline__ void mapped_residual(const DevArrays<R>& d, const Tab
             r[i] = s;
         }
     }
-    // faces
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-        const int kind = (inf >> (4 * f)) & 3;
-        if (kind == 0) continue;
-        const int k = f >> 1, sd = f & 1;
-        if (kind == 3) {
-            mapped_hanging_coarse<R, DIM, P>(d, T, tick, B, e, f, u, r);
-            continue;
+    // faces: the side a loop where the rows are not all in registers, the subfaces always (unrolled
+    // over 6 faces, 4 subfaces and 4 points the FP64 Q1 step was 700 KB of code, fetched from L2)
+    auto face = [&](int k, int sd, R* un) {
+        const int f = 2 * k + sd, kind = (inf >> (4 * f)) & 3;
+        if (kind == 0 || kind == 3) return;
+        if constexpr (!ALL) {
+            const int n = sd ? mt.nbf[2 * k + 1] : mt.nbf[2 * k];
+            const R* ol;
+            R th;
+            ld_dofs<R, NP, NPS>(seen_row<R, NPS>(d, tick, B, n, sd ? mt.lvn[2 * k + 1] : mt.lvn[2 * k], ol, th), un);
+            if (th > R(0)) interp_row<R, NP, NPS>(ol, th, un);
         }
-        R un[NP];
-        load_seen<R, NP, NPS>(d, tick, B, d.nbr[(size_t)e * NF + f], un);
         const R* bs = sd ? T.bR : T.bL;
         const R* ds = sd ? T.dR : T.dL;
         int tg[2] = {0, 0};
         face_tangents<DIM>(k, tg);
         R to[NPF], tn[NPF], flo[NPF], fln[NPF];
-        const R* gf = d.gface + ((size_t)e * NF + f) * NPF * FPV;
+        const R* gf = factors_of(d.gface, e, M::NFV) + f * NPF * FPV * FS;
         mapped_face_fluxes<R, DIM, P>(T, u, un, k, sd, gf, to, tn, flo, fln);
         if (kind == 2) {
             // a coarser neighbour: its trace and flux at this element's points, on the half of
@@ -284,14 +315,14 @@ __device__ __forceinline__ void mapped_residual(const DevArrays<R>& d, const Tab
             for (int t = 0; t < NPF; ++t) {
                 R L[2][P + 1], DL[2][P + 1];
                 half_rows<R, DIM, P>(T, t, pos, L, DL);
-                face_point_eval<R, DIM, P>(T, un, k, sd ^ 1, tg, L, DL, gf + t * FPV, R(0.5), tn[t], fln[t]);
+                face_point_eval<R, DIM, P>(T, un, k, sd ^ 1, tg, L, DL, gf + t * FPV * FS, R(0.5), tn[t], fln[t]);
             }
         }
 #pragma unroll
         for (int t = 0; t < NPF; ++t) {
             const int at[2] = {t % N1, t / N1};
-            const R* c = gf + t * FPV;
-            const R dS = c[DIM], kap = c[DIM + 1];
+            const R* c = gf + t * FPV * FS;
+            const R dS = c[DIM * FS], kap = c[(DIM + 1) * FS];
             const R jump = to[t] - tn[t];
             const R A = dS * (R(-0.5) * (flo[t] + fln[t]) + kap * jump);
             const R Bc = R(-0.5) * dS * jump;
@@ -300,29 +331,43 @@ __device__ __forceinline__ void mapped_residual(const DevArrays<R>& d, const Tab
 #pragma unroll
             for (int m = 0; m < N1; ++m) {
                 const int i = q0 + m * stride<N1>(k);
-                r[i] += A * bs[m] + Bc * c[k] * ds[m];
+                r[i] += A * bs[m] + Bc * c[k * FS] * ds[m];
 #pragma unroll
                 for (int z = 0; z < DIM - 1; ++z) {
-                    const R w = Bc * c[tg[z]] * bs[m];
+                    const R w = Bc * c[tg[z] * FS] * bs[m];
 #pragma unroll
                     for (int a = 0; a < N1; ++a) r[i + (a - at[z]) * stride<N1>(tg[z])] += w * T.D1[at[z]][a];
                 }
             }
         }
+    };
+    if constexpr (ALL) {
+#pragma unroll
+        for (int f = 0; f < NF; ++f) face(f >> 1, f & 1, un_[f]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < DIM; ++k)
+#pragma unroll 1
+            for (int sd = 0; sd < 2; ++sd) face(k, sd, un_[0]);
     }
+#pragma unroll
+    for (int k = 0; k < DIM; ++k)
+#pragma unroll 1
+        for (int sd = 0; sd < 2; ++sd)
+            if (((inf >> (8 * k + 4 * sd)) & 3) == 3) mapped_hanging_coarse<R, DIM, P>(d, T, tick, B, e, k, sd, u, r);
 }
 
 // One element step of Alg. 1 on a mapped mesh (see tick_elem for the box elements).
 template <typename R, int DIM, int P>
 __device__ __forceinline__ void tick_elem_mapped(const TickArgs<R>& a, const Tables<R>& T, const Phys<R>& ph,
-                                                 int tick, int e) {
+                                                 int tick, const TickMeta<DIM, P>& mt) {
     using M = MapShape<DIM, P>;
     constexpr int NP = M::NP, VPN = M::VPN;
     constexpr int NPS = Shape<DIM, P>::NPS;
     const DevArrays<R>& d = a.d;
-    const uint8_t lvb = d.lvl[e];
-    const uint32_t inf = d.info[e];
-    const int b = lvb & 7, par = (lvb >> 3) & 1;
+    const int e = mt.e;
+    const uint32_t inf = mt.inf;
+    const int b = mt.lv & 7, par = (mt.lv >> 3) & 1;
     const int ke = tick >> (a.B - b);
     const int cur = par ^ (ke & 1);
     const R* Vc = (cur ? d.V1 : d.V0) + (size_t)e * NPS;
@@ -331,7 +376,7 @@ __device__ __forceinline__ void tick_elem_mapped(const TickArgs<R>& a, const Tab
     R u[NP], w[NP], r[NP], Ia[NP], ga[NP];
     ld_dofs<R, NP, NPS>(Vc, u);
     ld_dofs<R, NP, NPS>(vp, w);
-    mapped_residual<R, DIM, P>(d, T, tick, a.B, e, inf, u, r);
+    mapped_residual<R, DIM, P>(d, T, tick, a.B, mt, u, r);
     double acc0 = 0.0;
     if (ke != 0) {
         ld_dofs<R, NP, NPS>(d.Ia + (size_t)e * NPS, Ia);
@@ -342,15 +387,33 @@ __device__ __forceinline__ void tick_elem_mapped(const TickArgs<R>& a, const Tab
     for (int s = 0; s < a.stim.n; ++s) stim = stim || d.smask[s][e] != 0u;
     const double dte_d = a.dte[b];
     const R dte = a.dteR[b];
-    const R* gv = d.gvol + (size_t)e * NP * VPN;
-    R un[NP], wn[NP];
+    StimMasks stm;
+    elem_stim<R>(a, e, stim ? INFO_STIM : 0u, tick, dte_d, stm);   // (info's bit is the box elements')
+    const R* gv = factors_of(d.gvol, e, M::NV);
+    R un[NP], wn[NP], Mq[NP], so[NP], sm[NP];
     R term = R(0), vmax = R(0);
 #pragma unroll
     for (int q = 0; q < NP; ++q) {
-        R so = R(0), sm = R(0);
-        if (stim) dof_stim<R>(a, e, tick, dte_d, q, so, sm);
-        const R Mq = gv[q * VPN + VPN - 1];
-        term += dof_update<R>(ph, Mq, R(1) / Mq, ke, dte, so, sm, u[q], w[q], r[q], Ia[q], ga[q], un[q], wn[q]);
+        Mq[q] = gv[(q * VPN + VPN - 1) * FS];
+        node_stim<R>(a, stm, q, so[q], sm[q]);
+    }
+    bool ap = false;
+    if constexpr (sizeof(R) == 4) {
+        ap = ph.ionic == 0 && ph.integrator == 1;
+        if (ap) {
+#pragma unroll
+            for (int q = 0; q < NP; ++q) r[q] *= R(1) / Mq[q];
+            term = ap_step<NP>(ApConst(ph), ke == 0, Mq, R(1), dte, so, sm, u, w, r, Ia, ga, un, wn);
+        }
+    }
+    if (!ap) {
+#pragma unroll
+        for (int q = 0; q < NP; ++q)
+            term += dof_update<R>(ph, Mq[q], R(1) / Mq[q], ke, dte, so[q], sm[q], u[q], w[q], r[q], Ia[q], ga[q], un[q],
+                                  wn[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
         const R av = un[q] < R(0) ? -un[q] : un[q];
         vmax = av > vmax ? av : vmax;
     }
@@ -402,20 +465,22 @@ __global__ void __launch_bounds__(128) k_eta_s_mapped(const DevArrays<R> d, cons
             acc += hF / (2.0 * P) * (double)sum;
         };
 #pragma unroll
-        for (int f = 0; f < NF; ++f) {
-            const int kind = (inf >> (4 * f)) & 3;
+        for (int k = 0; k < DIM; ++k)
+#pragma unroll 1
+        for (int sd = 0; sd < 2; ++sd) {
+            const int f = 2 * k + sd, kind = (inf >> (4 * f)) & 3;
             if (kind == 0) continue;
-            const int k = f >> 1, sd = f & 1;
             int tg[2] = {0, 0};
             face_tangents<DIM>(k, tg);
             const int nb = d.nbr[(size_t)e * NF + f];
             if (kind == 3) {
                 // the finer neighbours' subfaces, at their points with their factors
+#pragma unroll 1
                 for (int sb = 0; sb < (1 << (DIM - 1)); ++sb) {
                     const int j = d.hang[nb + sb];
                     R uj[NP];
                     ld_dofs<R, NP, NPS>((((d.lvl[j] >> 3) & 1) ? d.V1 : d.V0) + (size_t)j * NPS, uj);
-                    const R* gfj = d.gface + ((size_t)j * NF + (f ^ 1)) * NPF * FPV;
+                    const R* gfj = factors_of(d.gface, j, M::NFV) + (f ^ 1) * NPF * FPV * FS;
                     R tj[NPF], tx[NPF], fj[NPF], fx[NPF], dS[NPF], jmp[NPF];
                     mapped_face_fluxes<R, DIM, P>(T, uj, uj, k, sd ^ 1, gfj, tj, tx, fj, fx);
 #pragma unroll
@@ -423,9 +488,9 @@ __global__ void __launch_bounds__(128) k_eta_s_mapped(const DevArrays<R> d, cons
                         R L[2][P + 1], DL[2][P + 1];
                         half_rows<R, DIM, P>(T, t, sb, L, DL);
                         R tro, flo;
-                        face_point_eval<R, DIM, P>(T, u, k, sd, tg, L, DL, gfj + t * FPV, R(-0.5), tro, flo);
+                        face_point_eval<R, DIM, P>(T, u, k, sd, tg, L, DL, gfj + t * FPV * FS, R(-0.5), tro, flo);
                         jmp[t] = flo + fj[t];
-                        dS[t] = gfj[t * FPV + DIM];
+                        dS[t] = gfj[(t * FPV + DIM) * FS];
                     }
                     face_sum(dS, jmp);
                 }
@@ -433,7 +498,7 @@ __global__ void __launch_bounds__(128) k_eta_s_mapped(const DevArrays<R> d, cons
             }
             R un[NP];
             ld_dofs<R, NP, NPS>((((d.lvl[nb] >> 3) & 1) ? d.V1 : d.V0) + (size_t)nb * NPS, un);
-            const R* gf = d.gface + ((size_t)e * NF + f) * NPF * FPV;
+            const R* gf = factors_of(d.gface, e, M::NFV) + f * NPF * FPV * FS;
             R to[NPF], tn[NPF], flo[NPF], fln[NPF], dS[NPF], jmp[NPF];
             mapped_face_fluxes<R, DIM, P>(T, u, un, k, sd, gf, to, tn, flo, fln);
             if (kind == 2) {
@@ -442,13 +507,13 @@ __global__ void __launch_bounds__(128) k_eta_s_mapped(const DevArrays<R> d, cons
                 for (int t = 0; t < NPF; ++t) {
                     R L[2][P + 1], DL[2][P + 1];
                     half_rows<R, DIM, P>(T, t, pos, L, DL);
-                    face_point_eval<R, DIM, P>(T, un, k, sd ^ 1, tg, L, DL, gf + t * FPV, R(0.5), tn[t], fln[t]);
+                    face_point_eval<R, DIM, P>(T, un, k, sd ^ 1, tg, L, DL, gf + t * FPV * FS, R(0.5), tn[t], fln[t]);
                 }
             }
 #pragma unroll
             for (int t = 0; t < NPF; ++t) {
                 jmp[t] = flo[t] - fln[t];
-                dS[t] = gf[t * FPV + DIM];
+                dS[t] = gf[(t * FPV + DIM) * FS];
             }
             face_sum(dS, jmp);
         }
@@ -480,8 +545,7 @@ __device__ __forceinline__ int b_from_bound_dev(double dt, double bound) {
 // Factors of the current mesh after an adaptation, part 1.  An element kept by the adaptation
 // (pkind 0) with the face kinds it had takes its old factors, GL masses, signature (face kinds
 // in bits 0-11, level in bits 12-15, b^CFL in bits 16-19) and stimulus masks (source psrc in the
-// old set); a warp walks 32 consecutive elements and copies each kept element's factor rows with
-// its lanes (coalesced).  Every other element is appended to `todo` (count m->nfac, zeroed by
+// old set); a warp walks 32 consecutive elements.  Every other element is appended to `todo` (count m->nfac, zeroed by
 // the scan that commits the new mesh) for k_mapped_factors.  Without an old set (o* null)
 // every element is appended.
 template <typename R, int DIM, int P>
@@ -528,12 +592,18 @@ __global__ void __launch_bounds__(256) k_mapped_keep(
             slot = __shfl_sync(0xffffffffu, slot, 0);
             if ((need >> lane) & 1u) todo[slot + __popc(need & ((1u << lane) - 1u))] = (int32_t)e;
         }
-        for (unsigned kept = __ballot_sync(0xffffffffu, keep); kept; kept &= kept - 1u) {
-            const int l = __ffs(kept) - 1;
-            const int64_t ek = base + l, ok = __shfl_sync(0xffffffffu, o, l);
-            for (int i = lane; i < NV; i += 32) gvol[(size_t)ek * NV + i] = ogvol[(size_t)ok * NV + i];
-            for (int i = lane; i < NFV; i += 32) gface[(size_t)ek * NFV + i] = ogface[(size_t)ok * NFV + i];
-            for (int i = lane; i < NP; i += 32) mass[(size_t)ek * NP + i] = omass[(size_t)ok * NP + i];
+        if (keep) {
+            // lanes over the elements: the new places are consecutive, the old ones nearly so
+            const R* gvo = factors_of(ogvol, o, NV);
+            const R* gfo = factors_of(ogface, o, NFV);
+            R* gv = factors_of(gvol, e, NV);
+            R* gf = factors_of(gface, e, NFV);
+#pragma unroll 8
+            for (int i = 0; i < NV; ++i) gv[i * FS] = gvo[i * FS];
+#pragma unroll 8
+            for (int i = 0; i < NFV; ++i) gf[i * FS] = gfo[i * FS];
+#pragma unroll
+            for (int i = 0; i < NP; ++i) mass[(size_t)e * NP + i] = omass[(size_t)o * NP + i];
         }
     }
 }
@@ -557,7 +627,7 @@ struct GeoWarp {
 };
 
 // Returns the Gershgorin bound (every lane); writes the element's volume factors and GL masses
-// (gvol, gface, mass: the element's rows) and returns its stimulus masks in sk (every lane).
+// (gvol, gface: the element's factors, FS apart; mass: its row) and returns its stimulus masks in sk (every lane).
 // spt: CH * PS doubles and sm: NP doubles of shared memory owned by the warp.
 template <typename R, int DIM, int P>
 __device__ double geo_element_warp(const GeoArgs& g, const Tables<double>& T, const double* xg, const double* h0,
@@ -583,7 +653,7 @@ __device__ double geo_element_warp(const GeoArgs& g, const Tables<double>& T, co
     const int npt = off[NF];
     for (int f = 0; f < NF; ++f)
         if (kinds[f] == 0 || kinds[f] == 3)
-            for (int i = lane; i < NPF * FPV; i += 32) gface[f * NPF * FPV + i] = (R)0;
+            for (int i = lane; i < NPF * FPV; i += 32) gface[(f * NPF * FPV + i) * FS] = (R)0;
     uint32_t mk[MDL_MAX_STIM] = {0u, 0u, 0u, 0u};
     double bacc[NE];
 #pragma unroll
@@ -612,16 +682,16 @@ __device__ double geo_element_warp(const GeoArgs& g, const Tables<double>& T, co
                     K[i][j] = Wq * fabs(det) * s2h[i] * s * s2h[j];
                     rec[i * DIM + j] = K[i][j];
                 }
-            R* gv = gvol + q * VPN;
+            R* gv = gvol + q * VPN * FS;
             if (DIM == 2) {
-                gv[0] = (R)K[0][0]; gv[1] = (R)K[1][1]; gv[2] = (R)K[0][1];
+                gv[0] = (R)K[0][0]; gv[FS] = (R)K[1][1]; gv[2 * FS] = (R)K[0][1];
             } else {
-                gv[0] = (R)K[0][0]; gv[1] = (R)K[1][1]; gv[2] = (R)K[2][2];
-                gv[3] = (R)K[0][1]; gv[4] = (R)K[0][2]; gv[5] = (R)K[1][2];
+                gv[0] = (R)K[0][0]; gv[FS] = (R)K[1][1]; gv[2 * FS] = (R)K[2][2];
+                gv[3 * FS] = (R)K[0][1]; gv[4 * FS] = (R)K[0][2]; gv[5 * FS] = (R)K[1][2];
             }
             const double mq = Wq * fabs(det);
             mass[q] = mq;
-            gv[NS] = (R)mq;
+            gv[NS * FS] = (R)mq;
             sm[q] = mq;
             for (int s = 0; s < nstim; ++s) {
                 bool in = true;
@@ -664,10 +734,10 @@ __device__ double geo_element_warp(const GeoArgs& g, const Tables<double>& T, co
             const double dS = Wt * adet * ln;
             const double kap = g.gamma * nDn * ln / h[k] * pen;
             if (sb == 0 && kind != 3) {
-                R* gf = gface + (f * NPF + t) * FPV;
-                for (int i = 0; i < DIM; ++i) gf[i] = (R)c[i];
-                gf[DIM] = (R)dS;
-                gf[DIM + 1] = (R)kap;
+                R* gf = gface + (f * NPF + t) * FPV * FS;
+                for (int i = 0; i < DIM; ++i) gf[i * FS] = (R)c[i];
+                gf[DIM * FS] = (R)dS;
+                gf[(DIM + 1) * FS] = (R)kap;
             }
             double lt[2][3], dlt[2][3];
             for (int z = 0; z < nt; ++z) geo_lagrange<N1>(xg, xi_t[z], lt[z], dlt[z]);
@@ -787,8 +857,8 @@ __global__ void __launch_bounds__(64) k_mapped_factors(
         const int cc[3] = {c4.x, c4.y, c4.z};
         uint32_t sk[MDL_MAX_STIM] = {0u, 0u, 0u, 0u};
         const double cfl = geo_element_warp<R, DIM, P>(a.g, Td, a.xg, a.h0, c4.w, cc, kinds, a.nstim, a.slo, a.shi,
-                                                       s_pt[wib], s_m[wib], gvol + (size_t)e * NV,
-                                                       gface + (size_t)e * NFV, mass + (size_t)e * NP, sk);
+                                                       s_pt[wib], s_m[wib], factors_of(gvol, e, NV),
+                                                       factors_of(gface, e, NFV), mass + (size_t)e * NP, sk);
         if (lane == 0) {
             const int b = a.lts ? b_from_bound_dev(a.dt, cfl) : 0;
             bcfl[e] = (uint8_t)b;
@@ -800,11 +870,18 @@ __global__ void __launch_bounds__(64) k_mapped_factors(
 
 template <typename R, int DIM, int P>
 __global__ void __launch_bounds__(128) k_tick_mapped(const TickArgs<R> a, const Tables<R> T, const Phys<R> ph) {
+    // as k_tick: the due count and the first element's metadata before the dependent wait
     const int n_act = a.d.meta->nact[a.tick];
     const bool bad = a.d.meta->err != 0;
+    const int idx0 = (int)gtid();
+    TickMeta<DIM, P> m;
+    if (idx0 < n_act) tick_fetch<R, DIM, P>(a.d, idx0, m);
     pdl_enter();
     if (bad) return;
-    for (int idx = (int)gtid(); idx < n_act; idx += (int)gstride()) tick_elem_mapped<R, DIM, P>(a, T, ph, a.tick, a.d.order[idx]);
+    for (int idx = idx0; idx < n_act; idx += (int)gstride()) {
+        if (idx != idx0) tick_fetch<R, DIM, P>(a.d, idx, m);
+        tick_elem_mapped<R, DIM, P>(a, T, ph, a.tick, m);
+    }
 }
 
 }  // namespace mdl
