@@ -184,6 +184,33 @@ MDL_HD void face_map(const R (&A)[2][3][3], int c0, int c1, const R* in, R* out)
     }
 }
 
+// The transposes: out (+)= f A^T along tangent ti, out += (A_c0 x A_c1)^T in.
+template <typename R, int DIM, int P>
+MDL_HD void face_line_t(const R (&A)[3][3], int ti, R f, const R* in, R* out, bool add) {
+    using S = Shape<DIM, P>;
+    constexpr int N1 = S::N1;
+    const int st = ti == 0 ? 1 : N1;
+#pragma unroll
+    for (int t = 0; t < S::NT; ++t) {
+        const int tt = (t / st) % N1, base = t - tt * st;
+        R s = 0;
+#pragma unroll
+        for (int m = 0; m < N1; ++m) s += A[m][tt] * in[base + m * st];
+        out[t] = add ? out[t] + f * s : f * s;
+    }
+}
+template <typename R, int DIM, int P>
+MDL_HD void face_map_t_add(const R (&A)[2][3][3], int c0, int c1, const R* in, R* out) {
+    using S = Shape<DIM, P>;
+    if (DIM == 2) {
+        face_line_t<R, DIM, P>(A[c0], 0, R(1), in, out, true);
+    } else {
+        R t[S::NT];
+        face_line_t<R, DIM, P>(A[c0], 0, R(1), in, t, false);
+        face_line_t<R, DIM, P>(A[c1], 1, R(1), t, out, true);
+    }
+}
+
 // Mixed terms of a same-level or coarser neighbour: Xv = sum_l XF_kl C_l TN.
 template <typename R, int DIM, int P>
 MDL_HD void box_mixed(const BoxOp<R>& op, int k, int side, const R* TN, R* Xv) {

@@ -865,6 +865,58 @@ __device__ __forceinline__ float ap_step(const ApConst& c, const bool first, con
     return term;
 }
 
+static __device__ __noinline__ double expm1_call(double x) { return expm1(x); }   // (out of line: rarely taken)
+
+// e^x - 1 in FP64: the Taylor series of the exponential through x^8 for |x| < 2^-7 (truncation
+// below 1e-20 relative), else expm1.
+__device__ __forceinline__ double expm1_f64(double x) {
+    if (fabs(x) < 0.0078125)
+        return x * (1.0 + x * (0.5 + x * (1.0 / 6.0 + x * (1.0 / 24.0 + x * (1.0 / 120.0 + x * (1.0 / 720.0 +
+               x * (1.0 / 5040.0 + x * (1.0 / 40320.0))))))));
+    return expm1_call(x);
+}
+
+// The FP64 Aliev-Panfilov step of one DOF with the products shared as in ap_step, for either state
+// integrator: FP64 instructions issue at 1/64 of the FP32 rate, and the separate forms of I, g and
+// the state step took about 110 of them.  Returns mq [dI^2 + dg^2].
+__device__ __forceinline__ double ap_step_f64(const Phys<double>& ph, const bool first, double mq, double sc, double dte,
+                                              double so, double sm, double u, double w, double r, double& Ia,
+                                              double& ga, double& un, double& wn) {
+    const double a1 = ph.a + 1.0, it = ph.inv_ts, kt = ph.k * it;
+    auto eps_of = [&](double V, double s) {
+        double den = V + ph.mu2;
+        den = den > 1e-6 ? den : 1e-6;
+        return ph.eps0 + ph.mu1 * s / den;
+    };
+    const double q = u * (u - a1);
+    const double z = -ph.k * q - w;                                  // v_inf - w
+    const double I = u * (kt * (q + ph.a) + it * w) + so;
+    const double eps = eps_of(u, w) * it;
+    if (first) {
+        Ia = I;
+        ga = eps * z;
+    }
+    const double du = dte * (-r * sc - I);
+    const double dw = ph.integrator == 0 ? dte * eps * z : -z * expm1_f64(-eps * dte);
+    un = u + du;
+    wn = w + dw;
+    const double Vm = u + 0.5 * du, wm = w + 0.5 * dw;
+    const double qm = Vm * (Vm - a1);
+    const double dI = Vm * (kt * (qm + ph.a) + it * wm) + sm - Ia;
+    const double dg = eps_of(Vm, wm) * it * (-ph.k * qm - wm) - ga;
+    return mq * (dI * dI + dg * dg);
+}
+
+// dof_update through the shared forms where they apply.
+template <typename R>
+__device__ __forceinline__ R dof_update_any(const Phys<R>& ph, R Mq, R Minv, int ke, R dte, R so, R sm, R u, R w, R r,
+                                            R& Ia, R& ga, R& un, R& wn) {
+    if constexpr (sizeof(R) == 8) {
+        if (ph.ionic == 0) return ap_step_f64(ph, ke == 0, Mq, Minv, dte, so, sm, u, w, r, Ia, ga, un, wn);
+    }
+    return dof_update<R>(ph, Mq, Minv, ke, dte, so, sm, u, w, r, Ia, ga, un, wn);
+}
+
 // Pointwise part of one element step (Alg. 1) given the residual: Q1 r = (A u)_e (the GL
 // masses of an element are equal), Q2 rho = (M^-1 A u)_e in level-0 units (4^lev scales it); returns the element's RV-T term, vmax = max_q |V_new|.
 template <typename R, int DIM, int P>
@@ -896,7 +948,7 @@ __device__ __forceinline__ R elem_pointwise(const TickArgs<R>& a, const Phys<R>&
     for (int q = 0; q < NP; ++q) {
         R so, smd;
         node_stim<R>(a, stm, q, so, smd);
-        term += dof_update<R>(ph, ph.Wvol[lev] * op.wq[q], sc, ke, dte, so, smd, u[q], w[q], r[q], Ia[q], ga[q], un[q],
+        term += dof_update_any<R>(ph, ph.Wvol[lev] * op.wq[q], sc, ke, dte, so, smd, u[q], w[q], r[q], Ia[q], ga[q], un[q],
                               wn[q]);
         const R av = un[q] < R(0) ? -un[q] : un[q];
         vmax = av > vmax ? av : vmax;
@@ -963,7 +1015,7 @@ __device__ __forceinline__ R pointwise_q23(const TickArgs<R>& a, const Phys<R>& 
         if (!ap) {
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                term += dof_update<R>(ph, op.wq[4 * i + k], sc, ke, dte, so[k], smd[k], u[k], w[k], r[k], Ia[k],
+                term += dof_update_any<R>(ph, op.wq[4 * i + k], sc, ke, dte, so[k], smd[k], u[k], w[k], r[k], Ia[k],
                                       ga[k], un[k], wn[k]);
         }
 #pragma unroll

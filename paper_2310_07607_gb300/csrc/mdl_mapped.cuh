@@ -115,75 +115,74 @@ __device__ __forceinline__ void mapped_face_fluxes(const Tables<R>& T, const R* 
     }
 }
 
-// At a point of face (normal axis k, side sd) of an element with values v whose tangential basis
-// rows are L[z][m] and DL[z][m] (d/dxi of the element's own tangential coordinate): the trace and
-// cscale * c . grad_xi v.  Used where the point is not one of the element's own face GL points
-// (hanging faces: the coarse side at the fine points).
+// Trace and normal derivative of v at the nodes of its face (axis k, side sd).
 template <typename R, int DIM, int P>
-__device__ __forceinline__ void face_point_eval(const Tables<R>& T, const R* v, int k, int sd, const int* tg,
-                                                const R (*L)[P + 1], const R (*DL)[P + 1], const R* c, R cscale,
-                                                R& tr, R& fl) {
-    constexpr int N1 = P + 1;
+__device__ __forceinline__ void mapped_trace(const Tables<R>& T, int k, int sd, const R* v, R* tr, R* dn) {
+    using M = MapShape<DIM, P>;
     const R* bs = sd ? T.bR : T.bL;
     const R* ds = sd ? T.dR : T.dL;
-    R t = 0, gn = 0, g0 = 0, g1 = 0;
 #pragma unroll
-    for (int m = 0; m < N1; ++m)
+    for (int m = 0; m < M::NPF; ++m) {
+        R a = 0, b = 0;
 #pragma unroll
-        for (int m0 = 0; m0 < N1; ++m0)
-#pragma unroll
-            for (int m1 = 0; m1 < (DIM == 3 ? N1 : 1); ++m1) {
-                const int node = m * stride<N1>(k) + m0 * stride<N1>(tg[0]) + (DIM == 3 ? m1 * stride<N1>(tg[1]) : 0);
-                const R l1 = DIM == 3 ? L[1][m1] : R(1);
-                const R val = v[node];
-                t += bs[m] * L[0][m0] * l1 * val;
-                gn += ds[m] * L[0][m0] * l1 * val;
-                g0 += bs[m] * DL[0][m0] * l1 * val;
-                if (DIM == 3) g1 += bs[m] * L[0][m0] * DL[1][m1] * val;
-            }
-    tr = t;
-    fl = cscale * (c[k * FS] * gn + c[tg[0] * FS] * g0 + (DIM == 3 ? c[tg[1] * FS] * g1 : R(0)));
+        for (int j = 0; j < M::N1; ++j) {
+            const R x = v[line_node<DIM, P>(k, m, j)];
+            a += bs[j] * x;
+            b += ds[j] * x;
+        }
+        tr[m] = a;
+        dn[m] = b;
+    }
 }
 
-// r_i += A psi_i + Bc cscale c . grad_xi psi_i at such a point.
+// The coarse side of a hanging face at the finer side's GL points (half `bits` per tangent of its
+// own face), from its face's traces tr0 and normal derivatives dn0: the trace and cscale c . grad_xi,
+// c the flux vector stored at each point (FS apart).  One-dimensional interpolation, and derivatives
+// along the face from the interpolated trace (its own coordinate runs twice as fast): an eighth of
+// the operations of the sums over the element's nodes at every point, which the FP64 pipe bounds.
 template <typename R, int DIM, int P>
-__device__ __forceinline__ void face_point_distribute(const Tables<R>& T, int k, int sd, const int* tg,
-                                                      const R (*L)[P + 1], const R (*DL)[P + 1], const R* c, R cscale,
-                                                      R A, R Bc, R* r) {
-    constexpr int N1 = P + 1;
-    const R* bs = sd ? T.bR : T.bL;
-    const R* ds = sd ? T.dR : T.dL;
-    const R Bs = Bc * cscale;
+__device__ __forceinline__ void half_face_eval(const Tables<R>& T, const R* tr0, const R* dn0, int k, const int* tg,
+                                               int bits, const R* gf, R cscale, R* tr, R* fl) {
+    using M = MapShape<DIM, P>;
+    constexpr int NPF = M::NPF, FPV = M::FPV;
+    R dn[NPF];
+    face_map<R, DIM, P>(T.Pi, bits & 1, (bits >> 1) & 1, tr0, tr);
+    face_map<R, DIM, P>(T.Pi, bits & 1, (bits >> 1) & 1, dn0, dn);
 #pragma unroll
-    for (int m = 0; m < N1; ++m)
-#pragma unroll
-        for (int m0 = 0; m0 < N1; ++m0)
-#pragma unroll
-            for (int m1 = 0; m1 < (DIM == 3 ? N1 : 1); ++m1) {
-                const int node = m * stride<N1>(k) + m0 * stride<N1>(tg[0]) + (DIM == 3 ? m1 * stride<N1>(tg[1]) : 0);
-                const R l1 = DIM == 3 ? L[1][m1] : R(1);
-                const R psi = bs[m] * L[0][m0] * l1;
-                const R cg = c[k * FS] * ds[m] * L[0][m0] * l1 + c[tg[0] * FS] * bs[m] * DL[0][m0] * l1 +
-                             (DIM == 3 ? c[tg[1] * FS] * bs[m] * L[0][m0] * DL[1][m1] : R(0));
-                r[node] += A * psi + Bs * cg;
-            }
-}
-
-// Tangential basis rows at face point t of a half-face: the coarse side of a hanging face seen at
-// the finer side's GL point t, half `bits` (per tangent) of its own face.
-template <typename R, int DIM, int P>
-__device__ __forceinline__ void half_rows(const Tables<R>& T, int t, int bits, R (*L)[P + 1], R (*DL)[P + 1]) {
-    constexpr int N1 = P + 1;
-    const int at[2] = {t % N1, t / N1};
+    for (int t = 0; t < NPF; ++t) fl[t] = gf[(t * FPV + k) * FS] * dn[t];
 #pragma unroll
     for (int z = 0; z < DIM - 1; ++z) {
-        const int b = (bits >> z) & 1;
+        R g[NPF];
+        face_line<R, DIM, P>(T.D1, z, R(2), tr, g, false);
 #pragma unroll
-        for (int m = 0; m < N1; ++m) {
-            L[z][m] = T.Pi[b][at[z]][m];
-            DL[z][m] = T.Pd[b][at[z]][m];
-        }
+        for (int t = 0; t < NPF; ++t) fl[t] += gf[(t * FPV + tg[z]) * FS] * g[t];
     }
+#pragma unroll
+    for (int t = 0; t < NPF; ++t) fl[t] *= cscale;
+}
+
+// The adjoint: test values A and cscale Bc c . grad_xi at the points, added to the coefficients
+// trc, dnc of the coarse side's face traces and normal derivatives.
+template <typename R, int DIM, int P>
+__device__ __forceinline__ void half_face_adjoint(const Tables<R>& T, int k, const int* tg, int bits, const R* gf,
+                                                  R cscale, const R* A, const R* Bc, R* trc, R* dnc) {
+    using M = MapShape<DIM, P>;
+    constexpr int NPF = M::NPF, FPV = M::FPV;
+    R a[NPF], n[NPF];
+#pragma unroll
+    for (int t = 0; t < NPF; ++t) {
+        a[t] = A[t];
+        n[t] = cscale * Bc[t] * gf[(t * FPV + k) * FS];
+    }
+#pragma unroll
+    for (int z = 0; z < DIM - 1; ++z) {
+        R g[NPF];
+#pragma unroll
+        for (int t = 0; t < NPF; ++t) g[t] = cscale * Bc[t] * gf[(t * FPV + tg[z]) * FS];
+        face_line_t<R, DIM, P>(T.D1, z, R(2), g, a, true);
+    }
+    face_map_t_add<R, DIM, P>(T.Pi, bits & 1, (bits >> 1) & 1, a, trc);
+    face_map_t_add<R, DIM, P>(T.Pi, bits & 1, (bits >> 1) & 1, n, dnc);
 }
 
 // The faces of element e with finer neighbours (kind 3 on face f): each subface sb is the
@@ -201,29 +200,36 @@ __device__ __forceinline__ void mapped_hanging_coarse(const DevArrays<R>& d, con
     int tg[2] = {0, 0};
     face_tangents<DIM>(k, tg);
     const int base = d.nbr[(size_t)e * NF + f];
+    R tr0[NPF], dn0[NPF], trc[NPF], dnc[NPF];
+    mapped_trace<R, DIM, P>(T, k, sd, u, tr0, dn0);
+#pragma unroll
+    for (int t = 0; t < NPF; ++t) trc[t] = dnc[t] = R(0);
 #pragma unroll 1
     for (int sb = 0; sb < NSUB; ++sb) {
         const int j = d.hang[base + sb];
         R uj[NP];
         load_seen<R, NP, NPS>(d, tick, B, j, uj);
         const R* gfj = factors_of(d.gface, j, M::NFV) + (f ^ 1) * NPF * FPV * FS;
-        R tj[NPF], tx[NPF], fj[NPF], fx[NPF];
+        R tj[NPF], tx[NPF], fj[NPF], fx[NPF], tro[NPF], flo[NPF], A[NPF], Bc[NPF];
         mapped_face_fluxes<R, DIM, P>(T, uj, uj, k, sd ^ 1, gfj, tj, tx, fj, fx);
+        half_face_eval<R, DIM, P>(T, tr0, dn0, k, tg, sb, gfj, R(-0.5), tro, flo);
 #pragma unroll
         for (int t = 0; t < NPF; ++t) {
             const R* c = gfj + t * FPV * FS;
-            R L[2][P + 1], DL[2][P + 1];
-            half_rows<R, DIM, P>(T, t, sb, L, DL);
-            R tro, flo;
-            face_point_eval<R, DIM, P>(T, u, k, sd, tg, L, DL, c, R(-0.5), tro, flo);
             const R fln = -fj[t];
             const R dS = c[DIM * FS], kap = c[(DIM + 1) * FS];
-            const R jump = tro - tj[t];
-            const R A = dS * (R(-0.5) * (flo + fln) + kap * jump);
-            const R Bc = R(-0.5) * dS * jump;
-            face_point_distribute<R, DIM, P>(T, k, sd, tg, L, DL, c, R(-0.5), A, Bc, r);
+            const R jump = tro[t] - tj[t];
+            A[t] = dS * (R(-0.5) * (flo[t] + fln) + kap * jump);
+            Bc[t] = R(-0.5) * dS * jump;
         }
+        half_face_adjoint<R, DIM, P>(T, k, tg, sb, gfj, R(-0.5), A, Bc, trc, dnc);
     }
+    const R* bs = sd ? T.bR : T.bL;
+    const R* ds = sd ? T.dR : T.dL;
+#pragma unroll
+    for (int m = 0; m < NPF; ++m)
+#pragma unroll
+        for (int j = 0; j < M::N1; ++j) r[line_node<DIM, P>(k, m, j)] += bs[j] * trc[m] + ds[j] * dnc[m];
 }
 
 template <typename R, int DIM, int P>
@@ -310,13 +316,9 @@ __device__ __forceinline__ void mapped_residual(const DevArrays<R>& d, const Tab
         if (kind == 2) {
             // a coarser neighbour: its trace and flux at this element's points, on the half of
             // its face given by the position bits; its flux vector is half this element's
-            const int pos = (inf >> (4 * f + 2)) & 3;
-#pragma unroll
-            for (int t = 0; t < NPF; ++t) {
-                R L[2][P + 1], DL[2][P + 1];
-                half_rows<R, DIM, P>(T, t, pos, L, DL);
-                face_point_eval<R, DIM, P>(T, un, k, sd ^ 1, tg, L, DL, gf + t * FPV * FS, R(0.5), tn[t], fln[t]);
-            }
+            R trn[NPF], dnn[NPF];
+            mapped_trace<R, DIM, P>(T, k, sd ^ 1, un, trn, dnn);
+            half_face_eval<R, DIM, P>(T, trn, dnn, k, tg, (inf >> (4 * f + 2)) & 3, gf, R(0.5), tn, fln);
         }
 #pragma unroll
         for (int t = 0; t < NPF; ++t) {
@@ -409,7 +411,7 @@ __device__ __forceinline__ void tick_elem_mapped(const TickArgs<R>& a, const Tab
     if (!ap) {
 #pragma unroll
         for (int q = 0; q < NP; ++q)
-            term += dof_update<R>(ph, Mq[q], R(1) / Mq[q], ke, dte, so[q], sm[q], u[q], w[q], r[q], Ia[q], ga[q], un[q],
+            term += dof_update_any<R>(ph, Mq[q], R(1) / Mq[q], ke, dte, so[q], sm[q], u[q], w[q], r[q], Ia[q], ga[q], un[q],
                                   wn[q]);
     }
 #pragma unroll
@@ -475,21 +477,20 @@ __global__ void __launch_bounds__(128) k_eta_s_mapped(const DevArrays<R> d, cons
             const int nb = d.nbr[(size_t)e * NF + f];
             if (kind == 3) {
                 // the finer neighbours' subfaces, at their points with their factors
+                R tr0[NPF], dn0[NPF];
+                mapped_trace<R, DIM, P>(T, k, sd, u, tr0, dn0);
 #pragma unroll 1
                 for (int sb = 0; sb < (1 << (DIM - 1)); ++sb) {
                     const int j = d.hang[nb + sb];
                     R uj[NP];
                     ld_dofs<R, NP, NPS>((((d.lvl[j] >> 3) & 1) ? d.V1 : d.V0) + (size_t)j * NPS, uj);
                     const R* gfj = factors_of(d.gface, j, M::NFV) + (f ^ 1) * NPF * FPV * FS;
-                    R tj[NPF], tx[NPF], fj[NPF], fx[NPF], dS[NPF], jmp[NPF];
+                    R tj[NPF], tx[NPF], fj[NPF], fx[NPF], tro[NPF], flo[NPF], dS[NPF], jmp[NPF];
                     mapped_face_fluxes<R, DIM, P>(T, uj, uj, k, sd ^ 1, gfj, tj, tx, fj, fx);
+                    half_face_eval<R, DIM, P>(T, tr0, dn0, k, tg, sb, gfj, R(-0.5), tro, flo);
 #pragma unroll
                     for (int t = 0; t < NPF; ++t) {
-                        R L[2][P + 1], DL[2][P + 1];
-                        half_rows<R, DIM, P>(T, t, sb, L, DL);
-                        R tro, flo;
-                        face_point_eval<R, DIM, P>(T, u, k, sd, tg, L, DL, gfj + t * FPV * FS, R(-0.5), tro, flo);
-                        jmp[t] = flo + fj[t];
+                        jmp[t] = flo[t] + fj[t];
                         dS[t] = gfj[(t * FPV + DIM) * FS];
                     }
                     face_sum(dS, jmp);
@@ -502,13 +503,9 @@ __global__ void __launch_bounds__(128) k_eta_s_mapped(const DevArrays<R> d, cons
             R to[NPF], tn[NPF], flo[NPF], fln[NPF], dS[NPF], jmp[NPF];
             mapped_face_fluxes<R, DIM, P>(T, u, un, k, sd, gf, to, tn, flo, fln);
             if (kind == 2) {
-                const int pos = (inf >> (4 * f + 2)) & 3;
-#pragma unroll
-                for (int t = 0; t < NPF; ++t) {
-                    R L[2][P + 1], DL[2][P + 1];
-                    half_rows<R, DIM, P>(T, t, pos, L, DL);
-                    face_point_eval<R, DIM, P>(T, un, k, sd ^ 1, tg, L, DL, gf + t * FPV * FS, R(0.5), tn[t], fln[t]);
-                }
+                R trn[NPF], dnn[NPF];
+                mapped_trace<R, DIM, P>(T, k, sd ^ 1, un, trn, dnn);
+                half_face_eval<R, DIM, P>(T, trn, dnn, k, tg, (inf >> (4 * f + 2)) & 3, gf, R(0.5), tn, fln);
             }
 #pragma unroll
             for (int t = 0; t < NPF; ++t) {
