@@ -11,11 +11,11 @@
 //     back to back: the host waits for the device once, after the last.  Per class, the
 //     first rounds of the batch time every candidate on the batch itself -- launch shapes of
 //     the fused kernel (threads per block, due elements per work item) and "own sweeps"
-//     (each slot's own sweep variant on its own stream, e.g. the tensor-core sweep of a Q2
-//     3D FP32 slot) -- and keep the fastest.  A fused element takes the step of the
-//     thread-per-element sweep, so an instance gives the values it gives alone with that
-//     sweep up to the FP32 rounding of the two kernels' compilations; with own sweeps it
-//     gives the bits it gives alone.
+//     (each slot's own sweep variant on its own stream) -- and keep the fastest, counting what a
+//     fused round adds per slot.  A slot on its own runs its whole barrier as one graph.  A fused
+//     element takes the step of the thread-per-element sweep, so an instance gives the values it
+//     gives alone with that sweep up to the FP32 rounding of the two kernels' compilations; with
+//     own sweeps it gives the bits it gives alone.
 //   streams: every slot launches its own barriers (its own sweep variant) on its own
 //     stream before any is waited for, so their kernels overlap on the device; the sweep
 //     launch shape is tuned once per class on a temporary copy of the first admitted
@@ -160,6 +160,12 @@ constexpr int kFusedCands = (int)(sizeof(kFusedShapes) / sizeof(kFusedShapes[0])
 constexpr int kOwnCand = kFusedCands;
 constexpr int kCands = kFusedCands + 1;
 constexpr int kRoundsPerCand = 2;
+// What a fused round adds per slot beside its sweep: two graph launches instead of one and an event
+// with two stream waits on the host, and the join of the group's slots on the device.  Per round,
+// classes fused / all slots on their own: 8 small adapting requests 222 / 151 us, 24 mixed instances
+// 496 / 461 us, 8 of them 111 / 85 us, with sweeps of 0.13 ms fused against 0.20 to 0.28 ms own for
+// the 12 2D instances of the 24.
+constexpr double kFusedSlotMs = 0.03;
 
 int sm_count() {
     int dev = 0, n = 1;
@@ -408,12 +414,16 @@ int fused_complete(mdl_batch* b, const std::vector<char>& took_part, int64_t* to
         if ((int)g.cand_ms.size() < kCands) g.cand_ms.assign(kCands, 0.0);
         g.cand_ms[c] += ms;
         if (++g.tuned == kCands * kRoundsPerCand) {
+            // the fastest fused shape, unless the slots' own sweeps cost less with what a fused round
+            // adds per slot
             int best = 0;
-            for (int k = 1; k < kCands; ++k)
+            for (int k = 1; k < kFusedCands; ++k)
                 if (g.cand_ms[k] < g.cand_ms[best]) best = k;
-            g.own = best == kOwnCand;
+            const double extra = kFusedSlotMs * (double)g.members.size() * kRoundsPerCand;
+            g.own = g.cand_ms[kOwnCand] <= g.cand_ms[best] + extra;
+            const double least = *std::min_element(g.cand_ms.begin(), g.cand_ms.end());
             if (!g.own) g.shape = mdl::FusedShape{kFusedShapes[best][0], kFusedShapes[best][1], 0};
-            g.best_ms = g.cand_ms[best] / kRoundsPerCand;
+            g.best_ms = least / kRoundsPerCand;
             g.worst_ms = *std::max_element(g.cand_ms.begin(), g.cand_ms.end()) / kRoundsPerCand;
             g.own_ms = g.cand_ms[kOwnCand] / kRoundsPerCand;
             g.tuned = -1;

@@ -173,14 +173,17 @@ class Ctx : public CtxBase {
         int64_t cap = -1, launches = 0, ticks = 0;
     };
     PhaseGraph graphs[4][4][2];
+    PhaseGraph series[2];      // SERIES whole barriers, per state set at their start
     bool use_graphs = true;
     int tick_threads = 128, tick_bpsm = 16;   // sweep launch shape
     bool coop_sweep = false;                  // ticks + epilogue in one cooperative launch
     bool group_tick = false;                  // Q1: a group of (p+1)^d lanes per element
+    bool auto_sweep = true;                   // no variant asked for: small Q1 meshes take the groups too
     bool tensor_tick = false;                 // Q2 3D FP32: element residual on the tensor cores
     int sweep_blocks = 0;                     // bound on the tensor sweep's blocks (0: default)
     bool pdl = true;                          // programmatic dependent launch between kernels
     int64_t inflight = 0, inflight_start = 0; // barriers launched by begin_barriers
+    int64_t run_count = 0;                    // barriers launched since the graphs were dropped
 
     static int div_up(int64_t n, int64_t b) { return (int)((n + b - 1) / b); }
     // Launch a barrier-step kernel on the context's stream.  With pdl set, the launch
@@ -223,6 +226,17 @@ class Ctx : public CtxBase {
         while (threads > 32 && div_up(n, threads) < nsm) threads /= 2;
         return threads;
     }
+    // Whether a Q1 mesh is small enough for a lane per DOF: a step is then one chain of latencies,
+    // a quarter as long per lane (2D), and FP64 spreads over more SMs' pipes.  Per barrier step,
+    // thread / group: FP64 squares of 1024 elements 32.2 / 24.1 us, 4096 32.7 / 24.8, 9216 33.1 / 41.3;
+    // FP32 (16 ticks) 1600 elements 63 / 54 us, 3600 65 / 69; adapting FP32 requests of 160, 518 and
+    // 2005 elements 51.5 / 44.9, 82 / 74 and 114 / 96 us (all of the smallest capacity, 4096, by which
+    // an adapting mesh is judged).
+    bool small_groups() const {
+        const int64_t lanes = sweep_elems() * NP;
+        return lanes <= (int64_t)nsm * (pb.amr_enabled ? 256 : sizeof(R) == 8 ? 128 : 64);
+    }
+
     // Elements that a launch is sized for: the mesh's, or the capacity where it adapts.
     int64_t sweep_elems() const { return std::max<int64_t>(pb.amr_enabled ? cap : ne, 1); }
 
@@ -407,9 +421,9 @@ class Ctx : public CtxBase {
         init.nbar = nbar;
         init.cur_set = (unsigned)cs;
         MDL_CK(cudaMemcpyAsync(meta.p, &init, sizeof(DevMeta), cudaMemcpyHostToDevice, st));
+        ne = n;   // (the launches are sized for it)
         int rc = build_tables(cs, 1);
         if (rc) return rc;
-        ne = n;
         MDL_CK(cudaMemsetAsync(x.V0.p, 0, (size_t)n * NPS * sizeof(R), st));
         MDL_CK(cudaMemsetAsync(x.V1.p, 0, (size_t)n * NPS * sizeof(R), st));
         MDL_CK(cudaMemsetAsync(x.v.p, 0, (size_t)n * NPS * sizeof(R), st));
@@ -589,8 +603,9 @@ class Ctx : public CtxBase {
                 }
                 return MDL_OK;
             }
-            const int lanes = (P == 1 && group_tick) ? NP : 1;
-            const int tt = lanes > 1 ? tick_threads : spread_threads(sweep_elems(), tick_threads);
+            const bool grp = P == 1 && (group_tick || (auto_sweep && small_groups()));
+            const int lanes = grp ? NP : 1;
+            const int tt = spread_threads(sweep_elems() * lanes, tick_threads);
             const int gt = (int)std::min<int64_t>(div_up(sweep_elems() * lanes, tt),
                                                   (int64_t)nsm * tick_bpsm * (tick_threads / tt));
             if constexpr (tensor_capable) {
@@ -627,7 +642,7 @@ class Ctx : public CtxBase {
             for (int i = 0; i < nt; ++i) {
                 ta.tick = i;
                 if constexpr (P == 1) {
-                    if (group_tick) MDL_CK(launch_kx(pdl && i > 0, (k_tick_group<R, DIM>), gt, tt, ta, ph, T));
+                    if (grp) MDL_CK(launch_kx(pdl && i > 0, (k_tick_group<R, DIM>), gt, tt, ta, ph, T));
                     else MDL_CK(launch_kx(pdl && i > 0, (k_tick<R, DIM, P>), gt, tt, ta, T, ph, op));
                 } else {
                     MDL_CK(launch_kx(pdl && i > 0, (k_tick<R, DIM, P>), gt, tt, ta, T, ph, op));
@@ -662,6 +677,11 @@ class Ctx : public CtxBase {
         return ta;
     }
 
+    // Barriers in one graph for a context that steps many: one launch from the host, and the next
+    // barrier's first kernel follows the epilogue as the kernels of a barrier follow each other.
+    // Captured once SERIES_FROM barriers have run, so that a short run does not pay for it.
+    static constexpr int SERIES = 4, SERIES_FROM = 48;
+
     // The state set of phase ph_ of a barrier that starts on set o.
     int phase_set(int ph_, int o) const { return ph_ >= 2 && pb.amr_enabled ? (o ^ 1) : o; }
 
@@ -674,14 +694,19 @@ class Ctx : public CtxBase {
             return (int)MDL_OK;
         };
         if (direct || !use_graphs) return launch_all();
-        PhaseGraph& g = graphs[p0][p1][o];
+        return replay(graphs[p0][p1][o], launch_all);
+    }
+
+    // Replay a captured graph of what `launch` issues, capturing it first.
+    template <typename F>
+    int replay(PhaseGraph& g, F launch) {
         if (!g.exec || g.cap != cap) {
             if (g.exec) cudaGraphExecDestroy(g.exec);
             g.exec = nullptr;
             const int64_t kl0 = stats.kernel_launches, tl0 = stats.tick_launches;
             cudaGraph_t graph;
             MDL_CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-            int rc = launch_all();
+            int rc = launch();
             cudaError_t ec = cudaStreamEndCapture(st, &graph);
             if (rc) {
                 if (ec == cudaSuccess) cudaGraphDestroy(graph);
@@ -700,6 +725,34 @@ class Ctx : public CtxBase {
         MDL_CK(cudaGraphLaunch(g.exec, st));
         stats.kernel_launches += g.launches;
         stats.tick_launches += g.ticks;
+        return MDL_OK;
+    }
+
+    // n barriers, in series of SERIES where a graph of them pays.
+    int run_barriers(int64_t n) {
+        while (n > 0) {
+            const bool direct = ovr_levels || ovr_eta_s || ovr_eta_t;
+            if (n >= SERIES && !direct && !timing && use_graphs && run_count >= SERIES_FROM) {
+                const int o = cs;
+                static_assert(SERIES % 2 == 0, "a series ends on the state set it starts on");
+                const int rc = replay(series[o], [&]() {
+                    for (int i = 0, c = o; i < SERIES; ++i) {
+                        for (int p = first_phase(); p <= last_phase(); ++p)
+                            if (int r = launch_phase(p, phase_set(p, c))) return r;
+                        c = phase_set(2, c);
+                    }
+                    return (int)MDL_OK;
+                });
+                if (rc) return rc;
+                n -= SERIES;
+                run_count += SERIES;
+                continue;
+            }
+            const int rc = run_barrier();
+            if (rc) return rc;
+            --n;
+            ++run_count;
+        }
         return MDL_OK;
     }
 
@@ -743,6 +796,11 @@ class Ctx : public CtxBase {
                     if (g.exec) cudaGraphExecDestroy(g.exec);
                     g = PhaseGraph{};
                 }
+        for (auto& g : series) {
+            if (g.exec) cudaGraphExecDestroy(g.exec);
+            g = PhaseGraph{};
+        }
+        run_count = 0;
     }
 
     void collect_timing() {
@@ -792,6 +850,8 @@ public:
             const int rc = mapped_factors(pb, Td, &mf, &err);
             if (rc) return rc;
         }
+        std::vector<double> cfl1;    // bounds of the box element classes
+        if (pb.lts_enabled || (pb.dt_barrier <= 0 && !mapped)) class_cfl_level1(Td, phd, DIM, P, pb.max_refine, &cfl1);
         if (pb.dt_barrier > 0) {
             dt = pb.dt_barrier;
         } else if (mapped) {
@@ -802,7 +862,7 @@ public:
             while (ldexp(1.0, -k - B) > cmin) ++k;
             dt = ldexp(1.0, -k);
         } else {
-            dt = auto_dt_barrier(Td, phd, DIM, P, pb.max_refine, B);
+            dt = auto_dt_barrier(cfl1, DIM, pb.max_refine, B);
         }
         int dev = 0;
         MDL_CK(cudaGetDevice(&dev));
@@ -841,22 +901,13 @@ public:
         const size_t per = (size_t)1 << (2 * NF);
         std::vector<uint8_t> hcb((size_t)(pb.max_refine + 1) * per, 0);
         if (pb.lts_enabled) {
-            std::vector<double> vol, face;
-            for (int l = 0; l <= pb.max_refine; ++l) {
-                level_blocks(Td, phd, DIM, P, l, &vol, &face);
+            for (int l = 0; l <= pb.max_refine; ++l)
                 for (size_t cfg = 0; cfg < per; ++cfg) {
-                    bool valid = true;
-                    for (int f = 0; f < NF; ++f) {
-                        const unsigned kd = (cfg >> (2 * f)) & 3u;
-                        if ((kd == 2 && l == 0) || (kd == 3 && l == pb.max_refine)) valid = false;
-                    }
-                    if (!valid) continue;
-                    const double c = class_cfl_from_blocks(Td, phd, DIM, P, l, (unsigned)cfg, vol, face);
-                    int b = b_from_bound(dt, c);
+                    if (!class_admissible(DIM, l, pb.max_refine, (unsigned)cfg)) continue;
+                    int b = b_from_bound(dt, class_cfl(cfl1, l, (unsigned)cfg));
                     if (b < 0 || b > 15) b = 15;
                     hcb[l * per + cfg] = (uint8_t)b;
                 }
-            }
         }
         for (int q = 0; q < NP; ++q) {
             double w = 1.0;
@@ -1064,11 +1115,8 @@ public:
             // replayed indicators/levels apply to exactly one barrier: run it alone
             const bool ovr = ovr_levels || ovr_eta_s || ovr_eta_t;
             const int64_t chunk = ovr ? 1 : (n - done);
-            for (int64_t i = 0; i < chunk; ++i) {
-                int rc = run_barrier();
-                if (rc) return rc;
-            }
-            int rc = sync_meta();
+            int rc = run_barriers(chunk);
+            if (!rc) rc = sync_meta();
             if (rc) return rc;
             if (timing) {
                 stats.timed_barriers += (int64_t)pending_ev.size();
@@ -1121,10 +1169,7 @@ public:
         inflight_start = nbar;
         // replayed inputs apply to exactly one barrier
         if (ovr_levels || ovr_eta_s || ovr_eta_t) n = std::min<int64_t>(n, 1);
-        for (int64_t i = 0; i < n; ++i) {
-            int rc = run_barrier();
-            if (rc) return rc;
-        }
+        if (int rc = run_barriers(n)) return rc;
         inflight = n;
         return MDL_OK;
     }
@@ -1201,7 +1246,8 @@ public:
             return MDL_E_ARG;
         }
         const bool co = variant == MDL_SWEEP_COOP, gr = variant == MDL_SWEEP_GROUP, tn = variant == MDL_SWEEP_TENSOR;
-        if (co != coop_sweep || gr != group_tick || tn != tensor_tick) {
+        if (auto_sweep || co != coop_sweep || gr != group_tick || tn != tensor_tick) {
+            auto_sweep = false;
             coop_sweep = co;
             group_tick = gr;
             tensor_tick = tn;

@@ -1697,7 +1697,7 @@ __global__ void __launch_bounds__(256) k_tick_group(const TickArgs<R> a, const P
         for (int q = 1; q < NP; ++q)
             if (q == g) my_u = u[q];
         R un_g, wn_g;
-        R term = dof_update<R>(ph, sMq[lev * NP + g], sMinv[lev * NP + g], ke, a.dteR[b], so, smd, my_u, w, rg, Ia,
+        R term = dof_update_any<R>(ph, sMq[lev * NP + g], sMinv[lev * NP + g], ke, a.dteR[b], so, smd, my_u, w, rg, Ia,
                                ga, un_g, wn_g);
         R vmax = un_g < R(0) ? -un_g : un_g;
 #pragma unroll

@@ -4,6 +4,7 @@
 
 #include <math.h>
 
+#include <algorithm>
 #include <cmath>
 #include <stddef.h>
 #include <string.h>
@@ -309,36 +310,59 @@ void level_blocks(const Tables<double>& T, const Phys<double>& ph, int dim, int 
     else level_blocks_t<3, 2>(T, ph, level, vol->data(), face->data());
 }
 
-double class_cfl_from_blocks(const Tables<double>& T, const Phys<double>& ph, int dim, int p, int level,
-                             unsigned cfg, const std::vector<double>& vol, const std::vector<double>& face) {
+namespace {
+
+// Gershgorin bounds of every face configuration from the volume block and the faces' own blocks:
+// the own block accumulates face by face down the tree of configurations, so that a configuration
+// adds one face block to its parent's sum.
+struct ClassTree {
+    int nf, np, kinds;         // kinds 0 .. kinds - 1 of every face
+    const double* face;
+    const double* M;
+    double* out;
+    std::vector<double> B;     // the partial sums, one block per depth
+
+    void walk(int f, unsigned cfg) {
+        const int nn = np * np;
+        const double* Bf = B.data() + (size_t)f * nn;
+        if (f == nf) {
+            double worst = 0.0;
+            for (int i = 0; i < np; ++i) {
+                double q[27], row = 0.0;
+                for (int j = 0; j < np; ++j) q[j] = fabs(Bf[i * np + j]) / M[i];
+                for (int j = 0; j < np; ++j) row += q[j];
+                if (row > worst) worst = row;
+            }
+            out[cfg] = 1.0 / worst;
+            return;
+        }
+        double* Bn = B.data() + (size_t)(f + 1) * nn;
+        for (int kd = 0; kd < kinds; ++kd) {
+            const double* F = face + (size_t)(f * 4 + kd) * nn;
+            for (int i = 0; i < nn; ++i) Bn[i] = Bf[i] + F[i];
+            walk(f + 1, cfg | (unsigned)kd << (2 * f));
+        }
+    }
+};
+
+}  // namespace
+
+void class_cfl_level1(const Tables<double>& T, const Phys<double>& ph, int dim, int p, int L,
+                      std::vector<double>* cfl) {
     const int n1 = p + 1;
     const int NP = (dim == 2) ? n1 * n1 : n1 * n1 * n1;
-    std::vector<double> B(vol);
-    for (int f = 0; f < 2 * dim; ++f) {
-        const int kd = (cfg >> (2 * f)) & 3;
-        const double* F = face.data() + ((size_t)(f * 4 + kd) * NP) * NP;
-        for (int i = 0; i < NP * NP; ++i) B[i] += F[i];
-    }
-    double worst = 0.0;
+    std::vector<double> vol, face, M(NP);
+    level_blocks(T, ph, dim, p, 1, &vol, &face);
     for (int i = 0; i < NP; ++i) {
-        double Mi = ph.Wvol[level];
+        M[i] = ph.Wvol[1];
         int r = i;
-        for (int k = 0; k < dim; ++k) {
-            Mi *= T.w[r % n1];
-            r /= n1;
-        }
-        double row = 0.0;
-        for (int j = 0; j < NP; ++j) row += fabs(B[i * NP + j]) / Mi;
-        if (row > worst) worst = row;
+        for (int k = 0; k < dim; ++k, r /= n1) M[i] *= T.w[r % n1];
     }
-    return 1.0 / worst;
-}
-
-double class_cfl(const Tables<double>& T, const Phys<double>& ph, int dim, int p, int level,
-                 unsigned cfg) {
-    std::vector<double> vol, face;
-    level_blocks(T, ph, dim, p, level, &vol, &face);
-    return class_cfl_from_blocks(T, ph, dim, p, level, cfg, vol, face);
+    cfl->assign((size_t)1 << (4 * dim), 0.0);
+    ClassTree t{2 * dim, NP, L > 0 ? 4 : 2, face.data(), M.data(), cfl->data(), {}};
+    t.B.assign((size_t)(2 * dim + 1) * NP * NP, 0.0);
+    std::copy(vol.begin(), vol.end(), t.B.begin());
+    t.walk(0, 0u);
 }
 
 namespace {
@@ -528,30 +552,11 @@ int b_from_bound(double dt, double bound) {
     return -1;
 }
 
-double auto_dt_barrier(const Tables<double>& T, const Phys<double>& ph, int dim, int p, int L, int B) {
+double auto_dt_barrier(const std::vector<double>& cfl1, int dim, int L, int B) {
     double cmin = INFINITY;
-    const int nf = 2 * dim;
-    std::vector<double> vol, face;
-    for (int level = 0; level <= L; ++level) {
-        level_blocks(T, ph, dim, p, level, &vol, &face);
-        int choices[4], nc = 0;
-        choices[nc++] = 0;
-        choices[nc++] = 1;
-        if (level > 0) choices[nc++] = 2;
-        if (level < L) choices[nc++] = 3;
-        long total = 1;
-        for (int f = 0; f < nf; ++f) total *= nc;
-        for (long c = 0; c < total; ++c) {
-            unsigned cfg = 0;
-            long r = c;
-            for (int f = 0; f < nf; ++f) {
-                cfg |= (unsigned)choices[r % nc] << (2 * f);
-                r /= nc;
-            }
-            const double v = class_cfl_from_blocks(T, ph, dim, p, level, cfg, vol, face);
-            if (v < cmin) cmin = v;
-        }
-    }
+    for (int level = 0; level <= L; ++level)
+        for (size_t cfg = 0; cfg < cfl1.size(); ++cfg)
+            if (class_admissible(dim, level, L, (unsigned)cfg)) cmin = std::min(cmin, class_cfl(cfl1, level, (unsigned)cfg));
     int k = -20;
     while (ldexp(1.0, -k - B) > cmin) ++k;
     return ldexp(1.0, -k);

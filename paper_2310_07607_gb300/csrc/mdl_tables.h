@@ -1,6 +1,7 @@
 // mdl_tables.h -- host construction of basis tables, physics constants and CFL classes.
 #pragma once
 
+#include <math.h>
 #include <stdint.h>
 
 #include <vector>
@@ -24,16 +25,24 @@ template <typename R>
 void convert_phys(const Phys<double>& a, Phys<R>* b);
 
 // Gershgorin bound CFL_e = 1 / max_i (|L_ii| + sum_{j != i} |L_ij|), L = M^-1 K_e,
-// with K_e the element's own diagonal block of K = -A (Eq. cfl-monodomain), for an
-// element of `level` whose faces have kinds cfg (2 bits per face, FaceKind).
-double class_cfl(const Tables<double>& T, const Phys<double>& ph, int dim, int p, int level,
-                 unsigned cfg);
+// with K_e the element's own diagonal block of K = -A (Eq. cfl-monodomain), of a level-1
+// element for every set of face kinds cfg (2 bits per face, FaceKind).  On box elements L is
+// 4^l times its level-0 value, an exact scale, so that these are the bounds of every level.  On a
+// forest of depth L = 0 only those without coarser and finer neighbours.
+void class_cfl_level1(const Tables<double>& T, const Phys<double>& ph, int dim, int p, int L, std::vector<double>* cfl);
+inline double class_cfl(const std::vector<double>& cfl1, int level, unsigned cfg) { return ldexp(cfl1[cfg], 2 - 2 * level); }
+// Whether an element of `level` can have faces of kinds cfg on a forest of depth L.
+inline bool class_admissible(int dim, int level, int L, unsigned cfg) {
+    for (int f = 0; f < 2 * dim; ++f) {
+        const unsigned kd = (cfg >> (2 * f)) & 3u;
+        if ((kd == 2 && level == 0) || (kd == 3 && level == L)) return false;
+    }
+    return true;
+}
 // Per-level volume block and per (face, kind) own-side face blocks; the own block of a
 // class is vol + sum_f face[f][kind_f].
 void level_blocks(const Tables<double>& T, const Phys<double>& ph, int dim, int p, int level,
                   std::vector<double>* vol, std::vector<double>* face);
-double class_cfl_from_blocks(const Tables<double>& T, const Phys<double>& ph, int dim, int p, int level,
-                             unsigned cfg, const std::vector<double>& vol, const std::vector<double>& face);
 
 // Smallest b >= 0 with dt 2^-b <= bound; -1 if none below 60.
 int b_from_bound(double dt, double bound);
@@ -63,6 +72,7 @@ int q2_tensor_blocks(const Tables<double>& T, const Phys<double>& ph, std::vecto
 void q2_correction_blocks(const Tables<double>& T, const Phys<double>& ph, std::vector<float>* out);
 
 // Largest 2^-k with 2^-k 2^-B <= min over all admissible classes (levels 0..L).
-double auto_dt_barrier(const Tables<double>& T, const Phys<double>& ph, int dim, int p, int L, int B);
+// cfl1: class_cfl_level1.
+double auto_dt_barrier(const std::vector<double>& cfl1, int dim, int L, int B);
 
 }  // namespace mdl
