@@ -83,9 +83,9 @@ MDL_HD int line_node(int k, int m, int j) {
     return q;
 }
 
-// rho = own part.
+// rho = own part.  cross: op.cross != 0, which a kernel of its own for diagonal tensors knows.
 template <typename R, int DIM, int P>
-MDL_HD void box_own(const BoxOp<R>& op, const R* y, R* rho) {
+MDL_HD void box_own(const BoxOp<R>& op, const R* y, R* rho, bool cross) {
     using S = Shape<DIM, P>;
     constexpr int N1 = S::N1, NP = S::NP, NT = S::NT;
 #pragma unroll
@@ -100,7 +100,7 @@ MDL_HD void box_own(const BoxOp<R>& op, const R* y, R* rho) {
                 for (int j = 0; j < N1; ++j) s += op.S[k][a][j] * y[line_node<DIM, P>(k, m, j)];
                 rho[q] = s;
             }
-    if (op.cross) {
+    if (cross) {
 #pragma unroll
         for (int k = 0; k < DIM; ++k)
 #pragma unroll
@@ -241,7 +241,7 @@ MDL_HD void box_lift(const BoxOp<R>& op, int k, int side, const R* TN, const R* 
 // i = 0; finer: i = the subface) on the caller's shift.
 template <typename R, int DIM, int P, typename NB>
 MDL_HD void box_face_irregular(const BoxOp<R>& op, int k, int side, int kind, int pos, const R* y, NB nb, R* TN, R* DN,
-                               R* Xv) {
+                               R* Xv, bool cross) {
     using S = Shape<DIM, P>;
     constexpr int NT = S::NT, NP = S::NP;
     int tg[2] = {0, 0};
@@ -255,7 +255,7 @@ MDL_HD void box_face_irregular(const BoxOp<R>& op, int k, int side, int kind, in
             DN[m] = -dno[m];
             Xv[m] = R(0);
         }
-        if (op.cross) {
+        if (cross) {
             // no flux through the boundary: + s/2 D_kl (2/h_l) E_l times the own trace
 #pragma unroll
             for (int ti = 0; ti < DIM - 1; ++ti)
@@ -283,7 +283,7 @@ MDL_HD void box_face_irregular(const BoxOp<R>& op, int k, int side, int kind, in
         face_map<R, DIM, P>(op.PR[fine], c0, c1, dv, z);
 #pragma unroll
         for (int m = 0; m < NT; ++m) DN[m] += fd * z[m];
-        if (op.cross) {
+        if (cross) {
 #pragma unroll
             for (int ti = 0; ti < DIM - 1; ++ti)
                 face_line<R, DIM, P>(op.D1, ti, fx * op.XF[k][side][tg[ti]], t, dv, ti > 0);
@@ -292,7 +292,7 @@ MDL_HD void box_face_irregular(const BoxOp<R>& op, int k, int side, int kind, in
             for (int m = 0; m < NT; ++m) Xv[m] += z[m];
         }
     }
-    if (op.cross) {
+    if (cross) {
 #pragma unroll
         for (int ti = 0; ti < DIM - 1; ++ti)
             face_line<R, DIM, P>(op.Dt, ti, R(-0.5) * op.XF[k][side][tg[ti]], TN, Xv, true);

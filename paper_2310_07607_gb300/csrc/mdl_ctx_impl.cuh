@@ -627,13 +627,14 @@ class Ctx : public CtxBase {
             }
             if constexpr (tensor_capable) {
                 // resident blocks only: each walks its due elements, fetching metadata a step ahead
+                const auto kernel = op.cross ? k_tick_q23<DIM, P, true> : k_tick_q23<DIM, P, false>;
                 const int smem = q23::smem_bytes(tt);
                 int occ = 0;
-                MDL_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tick_q23<DIM, P>, tt, smem));
+                MDL_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, tt, smem));
                 const int gq = std::min(gt, nsm * std::max(1, occ));
                 for (int i = 0; i < nt; ++i) {
                     ta.tick = i;
-                    MDL_CK(launch_kxs(pdl && i > 0, (size_t)smem, (k_tick_q23<DIM, P>), gq, tt, ta, T, ph, op));
+                    MDL_CK(launch_kxs(pdl && i > 0, (size_t)smem, kernel, gq, tt, ta, T, ph, op));
                     MDL_LAUNCHED();
                     stats.tick_launches++;
                 }
@@ -962,7 +963,9 @@ public:
             MDL_CK(cudaMemcpy(tcC.p, hc.data(), hc.size() * sizeof(float), cudaMemcpyHostToDevice));
             MDL_CK(cudaFuncSetAttribute((k_tick_tc<DIM, P>), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         tc::SMEM_BYTES));
-            MDL_CK(cudaFuncSetAttribute((k_tick_q23<DIM, P>), cudaFuncAttributeMaxDynamicSharedMemorySize,
+            MDL_CK(cudaFuncSetAttribute((k_tick_q23<DIM, P, true>), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        q23::smem_bytes(256)));
+            MDL_CK(cudaFuncSetAttribute((k_tick_q23<DIM, P, false>), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         q23::smem_bytes(256)));
             MDL_CK(cudaFuncSetAttribute((k_eta_q23<DIM, P>), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         q23::eta_smem_bytes(128)));

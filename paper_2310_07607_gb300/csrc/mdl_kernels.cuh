@@ -607,7 +607,7 @@ __device__ __forceinline__ void box_residual(const DevArrays<R>& d, const BoxOp<
     R y[NP];
 #pragma unroll
     for (int q = 0; q < NP; ++q) y[q] = u[q] - c;
-    box_own<R, DIM, P>(op, y, rho);
+    box_own<R, DIM, P>(op, y, rho, op.cross != 0);
     bool irr = false;
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
@@ -657,7 +657,8 @@ __device__ __forceinline__ void box_residual(const DevArrays<R>& d, const BoxOp<
             for (int q = 0; q < NP; ++q) v[q] -= c;
         };
         R TN[NT], DN[NT], Xv[NT];
-        box_face_irregular<R, DIM, P>(op, f >> 1, f & 1, kind, (inf >> (4 * f + 2)) & 3, y, nb, TN, DN, Xv);
+        box_face_irregular<R, DIM, P>(op, f >> 1, f & 1, kind, (inf >> (4 * f + 2)) & 3, y, nb, TN, DN, Xv,
+                                       op.cross != 0);
         box_lift<R, DIM, P, true>(op, f >> 1, f & 1, TN, DN, Xv, rho);
     }
 }
@@ -675,7 +676,7 @@ __device__ __forceinline__ void box_residual_q23(const DevArrays<R>& d, const Bo
     R y[NP];
 #pragma unroll
     for (int q = 0; q < NP; ++q) y[q] = u[q] - c;
-    box_own<R, 3, 2>(op, y, rho);
+    box_own<R, 3, 2>(op, y, rho, op.cross != 0);
     auto row = [&](int n, uint8_t lv, R* v) {
         const R* o;
         R t;
@@ -710,7 +711,7 @@ __device__ __forceinline__ void box_residual_q23(const DevArrays<R>& d, const Bo
                     const int n = kind == 2 ? nbf : d.hang[nbf + sb];
                     row(n, kind == 2 ? lvn : d.lvl[n], v);
                 };
-                box_face_irregular<R, 3, 2>(op, k, side, kind, (fi >> 2) & 3, y, nb, TN, DN, Xv);
+                box_face_irregular<R, 3, 2>(op, k, side, kind, (fi >> 2) & 3, y, nb, TN, DN, Xv, op.cross != 0);
             }
             box_lift<R, 3, 2, true>(op, k, side, TN, DN, Xv, rho);
         }

@@ -84,7 +84,7 @@ __device__ __forceinline__ void fetch_levels(const DevArrays<float>& d, const Ne
 
 // (The bound of 384 threads gives 168 registers, three blocks of 128 threads per SM, without
 // spills; 128 registers spill and were 16% slower.)
-template <int DIM, int P>
+template <int DIM, int P, bool CROSS>
 __global__ void __launch_bounds__(384, 1) k_tick_q23(const TickArgs<float> a, const Tables<float> T,
                                                     const Phys<float> ph, const BoxOp<float> op) {
     static_assert(DIM == 3 && P == 2, "Q2 3D only");
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(384, 1) k_tick_q23(const TickArgs<float> a, co
 #pragma unroll
             for (int q = 0; q < NP; ++q) y[q] = t[q] - c;
         }
-        box_own<float, 3, 2>(op, y, rho);
+        box_own<float, 3, 2>(op, y, rho, CROSS);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             copy_wait<1>();
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(384, 1) k_tick_q23(const TickArgs<float> a, co
 #pragma unroll
                     for (int q = 0; q < NP; ++q) v[q] -= c;
                     box_trace<float, 3, 2>(op, k, 1 - side, v, TN, DN);
-                    if (op.cross) {
+                    if constexpr (CROSS) {
                         float Xv[NT];
                         box_mixed<float, 3, 2>(op, k, side, TN, Xv);
                         box_lift<float, 3, 2, true>(op, k, side, TN, DN, Xv, rho);
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(384, 1) k_tick_q23(const TickArgs<float> a, co
                         for (int q = 0; q < NP; ++q) v[q] -= c;
                     };
                     float Xv[NT];
-                    box_face_irregular<float, 3, 2>(op, k, side, kind, (fi >> 2) & 3, y, nb, TN, DN, Xv);
+                    box_face_irregular<float, 3, 2>(op, k, side, kind, (fi >> 2) & 3, y, nb, TN, DN, Xv, CROSS);
                     box_lift<float, 3, 2, true>(op, k, side, TN, DN, Xv, rho);
                 }
                 if (k == 2 && side == 0) {

@@ -1,0 +1,72 @@
+"""Barriers replayed several to a graph, and the lane-per-DOF sweep that small Q1 meshes take when no
+variant is asked for.
+
+A run in one call (graphs of four barriers after the first 48) must give the bits of the same run one
+barrier per call: the kernels and their order are the same.  The two Q1 sweeps sum the same terms in
+another order: 60 barriers of at most 4 substeps, each within a few roundings of the local terms --
+240 x 6e-8 = 1.4e-5 in FP32 (held to 2e-5 of the largest value), 240 x 1.1e-16 in FP64 (held to 1e-12).
+"""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mdl():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for -m gpu tests")
+    from paper_2310_07607_gb300 import build, mdl as M
+    build.build()
+    return M
+
+
+def problem(dim, order, precision, amr):
+    base = (13, 9, 1) if dim == 2 else (7, 4, 3)
+    h = (8.0 * 0.0078125 if dim == 2 else 4.0 * 0.015625) * order
+    ext = tuple(base[k] * h if k < dim else 1.0 for k in range(3))
+    tau = W.COMPLETED_TAU[(dim, order)]
+    return W.Problem(dim=dim, order=order, extent=ext, base=base, sigma_l=1.2, sigma_t=0.4,
+                     fibre=W.fibre_from_angle(0.6), gamma=10.0 * order * order,
+                     stimuli=[W.Stimulus((0.0, 0.0, 0.0), tuple(0.2 * e for e in ext), 1.0, 0.0, 1.0)],
+                     dt_barrier=0.0, max_refine=2 if amr else 0, n_lts_levels=3, tau_cell=0.5, tau_refine=tau[0],
+                     tau_coarsen=tau[1], state_integrator=W.STATE_EXP, precision=precision, amr_enabled=amr,
+                     lts_enabled=1)
+
+
+@pytest.mark.parametrize("dim,order,precision,amr", [(2, 1, 32, 1), (2, 2, 32, 1), (3, 1, 64, 1), (3, 2, 32, 1),
+                                                     (2, 1, 64, 0), (3, 2, 32, 0)])
+def test_series_of_barriers_give_the_bits_of_single_steps(mdl, dim, order, precision, amr):
+    p = problem(dim, order, precision, amr)
+    n = 119                                     # 48 one by one, 17 series of four, 3 more
+    a, b = mdl.Sim(p), mdl.Sim(p)
+    for _ in range(n):
+        a.step_barriers(1)
+    b.step_barriers(n)
+    assert a.time()[1] == b.time()[1] == n
+    for x, y in zip(a.read_mesh(), b.read_mesh()):
+        assert np.array_equal(x, y)
+    assert np.array_equal(a.read_V(), b.read_V()) and np.array_equal(a.read_state(), b.read_state())
+    assert np.array_equal(a.read_activation(), b.read_activation())
+    for k in ("dof_updates", "tick_launches", "kernel_launches", "amr_rebuilds", "integral_V"):
+        assert a.stats()[k] == b.stats()[k], k
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("dim,precision,amr", [(2, 32, 0), (2, 64, 0), (3, 32, 0), (2, 64, 1), (3, 64, 1)])
+def test_small_q1_default_sweep_matches_the_thread_sweep(mdl, dim, precision, amr):
+    p = problem(dim, 1, precision, amr)
+    a, b = mdl.Sim(p), mdl.Sim(p)
+    b.set_sweep_variant(mdl.SWEEP_THREAD)
+    a.step_barriers(60)
+    b.step_barriers(60)
+    assert np.array_equal(a.read_mesh()[1], b.read_mesh()[1])
+    tol = 2e-5 if precision == 32 else 1e-12
+    for x, y in ((a.read_V(), b.read_V()), (a.read_state(), b.read_state())):
+        assert np.abs(x - y).max() <= tol * max(np.abs(y).max(), 1e-30)
+    a.close()
+    b.close()
