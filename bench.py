@@ -3,8 +3,8 @@
 Default workload (the largest single-GPU configuration, HBM-resident): the 3D slab
 2 x 0.7 x 0.3 cm, 128x48x20 Q2 DG hexes, octree AMR to depth 3 driven by the Kelly
 indicator, 4 synchronous LTS levels, Aliev-Panfilov, transversely isotropic conductivity
-(1.2 / 0.3 mS/cm along x), FP32 bulk arithmetic with the element residual on the tcgen05
-tensor cores.  The synthetic initial state is a planar excitation front at mid-slab;
+(1.2 / 0.3 mS/cm along x), FP32 bulk arithmetic with the element operator as sums of
+one-dimensional lines.  The synthetic initial state is a planar excitation front at mid-slab;
 setup barriers let the AMR refine it to depth 3 (2.8M elements) before warm-up.
 `--workload slab2d` runs the 2D slab (2x2 cm, 256x256 Q1, AMR 3, LTS 4), `spiral2d` the
 temporal-adaptivity workload, `lv3d` the curved LV-like shell sector (mapped Q1 hexes,

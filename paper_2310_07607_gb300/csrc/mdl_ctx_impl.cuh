@@ -639,7 +639,7 @@ class Ctx : public CtxBase {
                     stats.tick_launches++;
                 }
                 return MDL_OK;
-            }
+            } else
             for (int i = 0; i < nt; ++i) {
                 ta.tick = i;
                 if constexpr (P == 1) {

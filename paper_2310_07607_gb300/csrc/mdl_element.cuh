@@ -341,60 +341,4 @@ MDL_HD void face_term_own(const Tables<R>& T, const Phys<R>& ph, int k, int s, i
     face_term<R, DIM, P>(T, ph, k, s, lo, cb_own, own, ln, -1, zero, lf, r);
 }
 
-// Kelly-type flux jump contribution of one (sub)face (Eq. dg-error-estimate):
-//   h_F/(2p) sum_t W_t (W_F [D grad phi . n])^2, h_F = |F|^(1/(d-1)), W_F = |F| / 2^(d-1).
-template <typename R, int DIM, int P>
-MDL_HD double face_kelly(const Tables<R>& T, const Phys<R>& ph, int k, int s, int lo, int cb_own,
-                         const R* own, int ln, int cb_nb, const R* nb, int lf) {
-    using S = Shape<DIM, P>;
-    constexpr int NT = S::NT;
-    R vo[NT], vn[NT], go[DIM][NT], gn[DIM][NT], W[NT];
-    face_eval<R, DIM, P>(T, ph.h2[lo], k, s, cb_own, own, vo, go);
-    face_eval<R, DIM, P>(T, ph.h2[ln], k, -s, cb_nb, nb, vn, gn);
-    face_weights<R, DIM, P>(T, ph, lf, k, W);
-    const double WF = (double)ph.Wface[lf][k];
-    const double area = WF * (double)(1 << (DIM - 1));
-    const double hF = (DIM == 2) ? area : sqrt(area);
-    double acc = 0;
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-        R fo = 0, fn = 0;
-#pragma unroll
-        for (int l = 0; l < DIM; ++l) {
-            fo += ph.D[k][l] * go[l][t];
-            fn += ph.D[k][l] * gn[l][t];
-        }
-        const double j = (double)(fo - fn) * WF;
-        acc += (double)W[t] * j * j;
-    }
-    return hF / (2.0 * P) * acc;
-}
-
-// face_kelly without its FP64 factor: sum_t W_t (D grad phi . n jump)^2 in the working
-// precision (FP32 on the device, where FP64 runs at a small fraction of the FP32 rate); the
-// caller multiplies by kfac = h_F/(2p) W_F^2 and accumulates the faces in FP64.
-template <typename R, int DIM, int P>
-MDL_HD R face_kelly_sum(const Tables<R>& T, const Phys<R>& ph, int k, int s, int lo, int cb_own, const R* own,
-                        int ln, int cb_nb, const R* nb, int lf) {
-    using S = Shape<DIM, P>;
-    constexpr int NT = S::NT;
-    R vo[NT], vn[NT], go[DIM][NT], gn[DIM][NT], W[NT];
-    face_eval<R, DIM, P>(T, ph.h2[lo], k, s, cb_own, own, vo, go);
-    face_eval<R, DIM, P>(T, ph.h2[ln], k, -s, cb_nb, nb, vn, gn);
-    face_weights<R, DIM, P>(T, ph, lf, k, W);
-    R acc = 0;
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-        R fo = 0, fn = 0;
-#pragma unroll
-        for (int l = 0; l < DIM; ++l) {
-            fo += ph.D[k][l] * go[l][t];
-            fn += ph.D[k][l] * gn[l][t];
-        }
-        const R j = fo - fn;
-        acc += W[t] * j * j;
-    }
-    return acc;
-}
-
 }  // namespace mdl

@@ -7,12 +7,13 @@
 //   v       [ne * NPS] Aliev-Panfilov recovery variable (element-local, in place)
 //   Ia, ga  [ne * NPS] I(u_a, t_a) and g(u_a) at the barrier start (only for S_e > 1)
 //                      (NPS: the row stride, NP rounded up to 28 for Q2 3D; pad value 0)
-//   lvl     [ne]       b_e (bits 0-2) | parity par_e (bit 3)
+//   lvl     [ne]       b_e (bits 0-2) | parity par_e (bit 3) | ordering class (bit 4)
 //   info    [ne]       4 bits per face: kind (0 bnd, 1 same, 2 coarser, 3 finer) | pos << 2;
 //                      bits 24-27 refinement level; bit 28 in a stimulus box; bit 29 probes pending
 //   nbr     [ne * 2d]  neighbour element (same/coarser) or first hang[] index (finer)
 //   hang    [*]        2^(d-1) fine neighbours per hanging face
-//   order   [ne]       element ids sorted by b descending: tick i updates a prefix
+//   order   [ne]       element ids sorted by b descending (regular elements first within a level
+//                      on 3D Q2 and curved meshes): tick i updates a prefix
 //   acc     [ne]       FP64 RV-T accumulator; eta_t, eta_s [ne] FP64
 //   lat     [n_probe]  FP64 activation time per probe (+INF pending)
 #pragma once
