@@ -55,20 +55,10 @@ WORKLOADS = {
 SETUP_BARRIERS = 5
 # DRAM bytes per launch of the dominant kernel (dram__bytes_read.sum + dram__bytes_write.sum)
 # from one ncu capture of the same build, averaged over the launches of a barrier step in
-# their proportion (tick 0 once, the finer ticks 7 times).  ncu replays each launch with
-# cold caches, so this is an upper bound on the live traffic.  Set to None whenever the
-# kernel changes until it is captured again.
-# Keyed by (workload, kernel) at the workload's own base grid.  3D slab: captured on the same
-# slab at a quarter of its x extent (base 32x48x20: the same 2,457,600 finest elements due at
-# ticks 1-7, the same level-1 and level-3 elements at tick 4), tick 0 scaled to the full slab's
-# 2,736,960 elements by the elements due.
-TRAFFIC_PER_LAUNCH = {
-    # 2D slab: the eight ticks of one barrier step
-    ("slab2d", "k_tick<float,2,1>"): 6.6640e6,
-    # curved LV-like slab at full size: the eight ticks of one barrier step
-    ("lv3d", "k_tick_mapped<float,3,1>"): 4.4873e7,
-    # 3D slab: the quarter slab's eight ticks, tick 0 and tick 4 scaled to the full slab
-}
+# their proportion, keyed by (workload, kernel) at the workload's own base grid.  ncu replays
+# each launch with cold caches, so this is an upper bound on the live traffic.  An entry is
+# dropped when its kernel changes until it is captured again: none holds for the present kernels.
+TRAFFIC_PER_LAUNCH = {}
 # Mapped Q1 3D (lv3d): per element step the state 128 B, metadata and the RV-T accumulator
 # 49 B, and the element's geometric factors (8 nodes x 7 values + 6 faces x 4 points x 5
 # values, FP32) 704 B, over 8 DOFs: 110.1 B.
