@@ -911,12 +911,9 @@ public:
                 }
         }
         for (int q = 0; q < NP; ++q) {
-            double w = 1.0;
-            for (int k = 0; k < DIM; ++k) w *= Td.w[digit<N1>(q, k)];
-            epiw.wh[q] = (float)w;
-            epiw.wl[q] = (float)(w - (double)epiw.wh[q]);
+            epiw.w[q] = phd.Wvol[0];
+            for (int k = 0; k < DIM; ++k) epiw.w[q] *= Td.w[digit<N1>(q, k)];
         }
-        epiw.w0 = phd.Wvol[0];
         std::vector<double> hm(8 * NP);
         for (int l = 0; l < 8; ++l)
             for (int q = 0; q < NP; ++q) {

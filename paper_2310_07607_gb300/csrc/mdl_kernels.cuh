@@ -1406,24 +1406,10 @@ __device__ __forceinline__ double sqrt_seeded(double a) {
     return fma(fma(-s, s, a), h, s);
 }
 
-// Sum as an unevaluated pair of FP32 values: s + c with |c| at most an ulp of s, 48 bits together.
-struct Pair {
-    float s, c;
-    // += w x, w = wh + wl
-    __device__ __forceinline__ void add(float wh, float wl, float x) {
-        const float p = wh * x;
-        const float e = fmaf(wl, x, fmaf(wh, x, -p));       // the product's rounding and the weight's tail
-        const float t = s + p, z = t - s;
-        c += ((s - (t - z)) + (p - z)) + e;                 // the sum's rounding
-        s = t;
-    }
-};
-
-// Weights of int V on box elements: GL weight products as pairs (0 past the last node) and the
-// level-0 volume factor; level l scales by 2^(-d l), exact.
+// Weights of int V on box elements of level 0: GL weight products times the volume factor (0 past the
+// last node).  Level l scales them by 2^(-d l), exact.
 struct EpiWeights {
-    float wh[28], wl[28];
-    double w0;
+    double w[28];
 };
 
 __device__ __forceinline__ double warp_sum(double x) {
@@ -1444,33 +1430,40 @@ __device__ __forceinline__ double block_sum(double x) {
 }
 
 // Barrier epilogue: eta^t = sqrt(acc)/dt, parity flip of single-step elements, non-finite
-// check, per-block partial sums of int V = sum_q M_q V_q.  FP64 sums bound it (1.25 TFLOP/s: 0.3 ms
-// for 2.6M Q2 elements, two FP64 instructions a DOF), so FP32 contexts on box elements sum pairs of
-// FP32 values with the FP64 precision's weights; the threads' sums are FP64.  Rows of 27 values are
-// read by whole warps (see mdl_q23.cuh), shorter ones by their element's thread.
+// check, per-block partial sums of int V = sum_q M_q V_q in FP64, in either precision of the field.
+// The FP64 pipe bounds it (1.25 TFLOP/s; a conversion and a multiply-add a DOF): sums in pairs of
+// FP32 values took 0.21 ms less of a 6.2 ms barrier step on 2.79 M Q2 3D elements, but their error
+// grows with the elements a thread takes (3e-13 of the integral of a constant field at nine).  FP32
+// rows of 27 values are read by whole warps (see mdl_q23.cuh): a lane holds four consecutive values of
+// a row and adds their weighted sum; shorter rows, FP64 ones and those of curved elements
+// (per-element masses) are read by their element's thread.
 template <typename R, int DIM, int P>
 __global__ void __launch_bounds__(256) k_epilogue(const DevArrays<R> d, const double* __restrict__ mtab,
                                                  const EpiWeights ew, double dt, double inv_dt, int inv_dt_exact,
                                                  int mass_per_elem) {
-    pdl_enter();
     using S = Shape<DIM, P>;
     constexpr int NP = S::NP, NPS = S::NPS;
-    constexpr bool PAIRS = sizeof(R) == 4, COOP = PAIRS && NPS != NP;
+    constexpr bool F32 = sizeof(R) == 4, COOP = F32 && NPS != NP;
+    __shared__ double sw[28];
+    if (COOP) {
+        if (threadIdx.x < 28) sw[threadIdx.x] = ew.w[threadIdx.x];
+        __syncthreads();
+    }
+    pdl_enter();
     if (d.meta->err) return;
     const int64_t ne = d.meta->ne;
     double loc = 0.0;
-    Pair sum{0.0f, 0.0f};
     float nf = 0.0f;                 // not 0 once a value was not finite
     const int lane = threadIdx.x & 31;
     for (int64_t base = gtid() - lane; base < ne; base += gstride()) {
         const int64_t e = base + lane;
         const bool in = e < ne;
         uint8_t lv = 0;
-        int lev = 0;
+        int lev = -1;
         if (in) {
             // eta^t = sqrt(acc) / dt in FP64 (it sets b^cell); the product with 1/dt equals the
             // quotient whenever dt is a power of two, as the automatic barrier step is
-            const double a = d.acc[e], r = PAIRS ? sqrt_seeded(a) : sqrt(a);
+            const double a = d.acc[e], r = F32 ? sqrt_seeded(a) : sqrt(a);
             d.eta_t[e] = inv_dt_exact ? r * inv_dt : r / dt;
             lv = d.lvl[e];
             if ((lv & 7) == 0) {
@@ -1483,17 +1476,15 @@ __global__ void __launch_bounds__(256) k_epilogue(const DevArrays<R> d, const do
         const R* w = d.v + (size_t)(in ? e : base) * NPS;
         if (COOP && !mass_per_elem) {
             if constexpr (COOP) {
-                const float sl = in ? pow2_neg<float>(DIM * lev) : 0.0f;
 #pragma unroll
                 for (int j = 0; j < 7; ++j) {
                     const int t = 32 * j + lane, r = t / 7, c = t - 7 * r;
                     const float4 x = reinterpret_cast<const float4*>(__shfl_sync(0xffffffffu, (long long)Vc, r))[c];
                     const float4 y = reinterpret_cast<const float4*>(__shfl_sync(0xffffffffu, (long long)w, r))[c];
-                    const float sr = __shfl_sync(0xffffffffu, sl, r);
-                    sum.add(ew.wh[4 * c], ew.wl[4 * c], sr * x.x);
-                    sum.add(ew.wh[4 * c + 1], ew.wl[4 * c + 1], sr * x.y);
-                    sum.add(ew.wh[4 * c + 2], ew.wl[4 * c + 2], sr * x.z);
-                    sum.add(ew.wh[4 * c + 3], ew.wl[4 * c + 3], sr * x.w);
+                    const int lr = __shfl_sync(0xffffffffu, lev, r);
+                    const double sum = sw[4 * c] * (double)x.x + sw[4 * c + 1] * (double)x.y +
+                                       sw[4 * c + 2] * (double)x.z + sw[4 * c + 3] * (double)x.w;
+                    if (lr >= 0) loc += pow2_neg<double>(DIM * lr) * sum;
                     nf += 0.0f * x.x + 0.0f * x.y + 0.0f * x.z + 0.0f * x.w;
                     nf += 0.0f * y.x + 0.0f * y.y + 0.0f * y.z + 0.0f * y.w;
                 }
@@ -1502,22 +1493,15 @@ __global__ void __launch_bounds__(256) k_epilogue(const DevArrays<R> d, const do
             R x[NP], y[NP];
             ld_dofs<R, NP, NPS>(Vc, x);
             ld_dofs<R, NP, NPS>(w, y);
-            if (PAIRS && !mass_per_elem) {
-                const float sl = pow2_neg<float>(DIM * lev);
+            // GL masses: per (level, node) on box elements, per (element, node) on mapped ones
+            const double* Mq = mtab + (mass_per_elem ? (size_t)e * NP : (size_t)lev * NP);
 #pragma unroll
-                for (int q = 0; q < NP; ++q) sum.add(ew.wh[q], ew.wl[q], sl * (float)x[q]);
-            } else {
-                // GL masses: per (level, node) on box elements, per (element, node) on mapped ones
-                const double* Mq = mtab + (mass_per_elem ? (size_t)e * NP : (size_t)lev * NP);
-#pragma unroll
-                for (int q = 0; q < NP; ++q) loc += Mq[q] * (double)x[q];
-            }
-#pragma unroll
-            for (int q = 0; q < NP; ++q)
+            for (int q = 0; q < NP; ++q) {
+                loc += Mq[q] * (double)x[q];
                 if (!isfinite(x[q]) || !isfinite(y[q])) nf = 1.0f;
+            }
         }
     }
-    if (PAIRS && !mass_per_elem) loc = ((double)sum.s + (double)sum.c) * ew.w0;
     if (!(nf == 0.0f)) atomicOr(&d.meta->nf_pending, 1u);
     loc = block_sum(loc);
     __shared__ bool last;
