@@ -167,10 +167,11 @@ class Ctx : public CtxBase {
     std::vector<EvSet> pending_ev;
     mdl_stats stats{};
     // captured graphs of consecutive phases, per first and last phase and state set (an adapting
-    // barrier swaps sets)
+    // barrier swaps sets), with the capacity (the buffers) and the element count (the launch
+    // shapes and the sweep's kernel) that they were captured for
     struct PhaseGraph {
         cudaGraphExec_t exec = nullptr;
-        int64_t cap = -1, launches = 0, ticks = 0;
+        int64_t cap = -1, elems = -1, launches = 0, ticks = 0;
     };
     PhaseGraph graphs[4][4][2];
     PhaseGraph series[2];      // SERIES whole barriers, per state set at their start
@@ -701,7 +702,7 @@ class Ctx : public CtxBase {
     // Replay a captured graph of what `launch` issues, capturing it first.
     template <typename F>
     int replay(PhaseGraph& g, F launch) {
-        if (!g.exec || g.cap != cap) {
+        if (!g.exec || g.cap != cap || g.elems != sweep_elems()) {
             if (g.exec) cudaGraphExecDestroy(g.exec);
             g.exec = nullptr;
             const int64_t kl0 = stats.kernel_launches, tl0 = stats.tick_launches;
@@ -722,6 +723,7 @@ class Ctx : public CtxBase {
             stats.kernel_launches = kl0;
             stats.tick_launches = tl0;
             g.cap = cap;
+            g.elems = sweep_elems();
         }
         MDL_CK(cudaGraphLaunch(g.exec, st));
         stats.kernel_launches += g.launches;

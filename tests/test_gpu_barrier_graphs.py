@@ -70,3 +70,32 @@ def test_small_q1_default_sweep_matches_the_thread_sweep(mdl, dim, precision, am
         assert np.abs(x - y).max() <= tol * max(np.abs(y).max(), 1e-30)
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+def test_an_uploaded_mesh_runs_as_in_a_new_context(mdl, precision):
+    """900 root elements, then 3600 uploaded within the capacity, then 900 again: launch shapes and the
+    choice of the sweep follow the mesh that is stepped, not the one that was stepped before it."""
+    p = problem(2, 1, precision, 0).replace(base=(30, 30, 1), extent=(1.9, 1.9, 1.0), max_refine=1, stimuli=[],
+                                            dt_barrier=2.0 ** -8)
+
+    def mesh(level):
+        n = 30 << level
+        block = 1 << level                       # leaves in root order, then Morton order
+        xy = [(i * block + a, j * block + b) for j in range(30) for i in range(30)
+              for b in range(block) for a in range(block)]
+        assert len(xy) == n * n
+        return np.full(n * n, level, np.int8), np.array(xy, np.int32)
+
+    used = mdl.Sim(p)
+    for level in (0, 1, 0):
+        V = 0.5 + 0.5 * np.sin(np.arange((900 << (2 * level)) * 4) / 91.0)
+        new = mdl.Sim(p)
+        for g in (used, new):
+            g.upload_mesh(*mesh(level))
+            g.set_initial(V, 0.3 * V)
+            g.step_barriers(60)
+        assert np.array_equal(used.read_V(), new.read_V()) and np.array_equal(used.read_state(), new.read_state())
+        assert np.array_equal(used.read_indicators()[1], new.read_indicators()[1])
+        new.close()
+    used.close()
