@@ -240,8 +240,10 @@ int mdl_set_tick_shape(mdl_ctx* ctx, int32_t threads, int32_t blocks_per_sm);
 /* Sweep kernel variant.  All follow Alg. 1 tick by tick; THREAD and COOP run the same
  * per-element arithmetic, GROUP sums the face terms in another order; they agree to the
  * working precision's rounding:
- *   MDL_SWEEP_THREAD  one thread per due element, one launch per tick; the default (small Q1
- *                     meshes take GROUP until a variant is set);
+ *   MDL_SWEEP_THREAD  one thread per due element, one launch per tick; the default, except
+ *                     that until a variant is set Q1 contexts take GROUP if they are small (by
+ *                     DOFs per SM): in FP64 by their elements, or their roots where they
+ *                     adapt, in FP32 by their roots and only where they adapt;
  *   MDL_SWEEP_GROUP   Q1 only: (p+1)^d lanes per element, one lane per face and per DOF,
  *                     one launch per tick (Q2 contexts use MDL_SWEEP_THREAD);
  *   MDL_SWEEP_COOP    every tick and the barrier epilogue in one cooperative launch with

@@ -227,15 +227,28 @@ class Ctx : public CtxBase {
         while (threads > 32 && div_up(n, threads) < nsm) threads /= 2;
         return threads;
     }
-    // Whether a Q1 mesh is small enough for a lane per DOF: a step is then one chain of latencies,
-    // a quarter as long per lane (2D), and FP64 spreads over more SMs' pipes.  Per barrier step,
-    // thread / group: FP64 squares of 1024 elements 32.2 / 24.1 us, 4096 32.7 / 24.8, 9216 33.1 / 41.3;
-    // FP32 (16 ticks) 1600 elements 63 / 54 us, 3600 65 / 69; adapting FP32 requests of 160, 518 and
-    // 2005 elements 51.5 / 44.9, 82 / 74 and 114 / 96 us (all of the smallest capacity, 4096, by which
-    // an adapting mesh is judged).
+    int64_t n_root() const {
+        int64_t n = 1;
+        for (int k = 0; k < DIM; ++k) n *= pb.base[k];
+        return n;
+    }
+
+    // Whether a Q1 context takes a lane per DOF (k_tick_group) where no variant is asked for: a step is
+    // then one chain of latencies, shorter per lane, and FP64 spreads over more SMs' pipes.  The two
+    // kernels round differently, so an adapting context decides by its roots, which stay (its capacity
+    // and its leaves do not), a fixed one by its mesh.  Per barrier step, thread / group, in us:
+    //   FP64     fixed 2D, one level, 4096 elements 32.1 / 24.9, 4900 33.4 / 37.7 (the lanes' second
+    //            wave); 5 levels 327 / 185, 325 / 267; fixed 3D 2040 elements 74.1 / 34.7; adapting
+    //            2D of 4096 roots 132 / 98, 3D of 2040 169 / 93.  (Adapting meshes gain further on, 3D
+    //            of 7488 roots 143 / 122, but take the same line.)
+    //   FP32     fixed meshes lose, 3D at every size (1200 elements 34.0 / 40.7), 2D but for 3 levels
+    //            (2304 elements 30.7 / 28.8; 4 levels 35.7 / 42.6; spirals of 1600 63.2 / 71.8);
+    //            adapting to depth 2, 2D of 2916 roots 46.3 / 45.4, 4096 45.3 / 45.8, 3D of 2040 47.3 / 44.4,
+    //            3360 45.8 / 47.3; to depth 3, where a root holds more leaves, 2D of 576 73 / 65, 1600
+    //            64.5 / 64.0, 4096 65.6 / 67.2, 24 x 160 roots along the front 83 / 97.
     bool small_groups() const {
-        const int64_t lanes = sweep_elems() * NP;
-        return lanes <= (int64_t)nsm * (pb.amr_enabled ? 256 : sizeof(R) == 8 ? 128 : 64);
+        if (sizeof(R) == 8) return (pb.amr_enabled ? n_root() : ne) * NP <= (int64_t)nsm * 128;
+        return pb.amr_enabled && n_root() * NP <= ((int64_t)nsm * 108 >> std::max(0, pb.max_refine - 2));
     }
 
     // Elements that a launch is sized for: the mesh's, or the capacity where it adapts.

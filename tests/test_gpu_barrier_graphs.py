@@ -99,3 +99,75 @@ def test_an_uploaded_mesh_runs_as_in_a_new_context(mdl, precision):
         assert np.array_equal(used.read_indicators()[1], new.read_indicators()[1])
         new.close()
     used.close()
+
+
+# roots (adapting) or elements (fixed) at both sides of the line between the two Q1 sweeps: DOFs per SM
+@pytest.mark.parametrize("dim,precision,amr,depth,dofs_per_sm", [(2, 64, 0, 0, 128), (3, 64, 0, 0, 128), (2, 64, 1, 2, 128),
+                                                                (2, 32, 1, 2, 108), (3, 32, 1, 2, 108), (2, 32, 1, 3, 54),
+                                                                (2, 32, 0, 0, 0), (3, 32, 0, 0, 0)])
+def test_default_q1_sweep_is_the_one_stated(mdl, dim, precision, amr, depth, dofs_per_sm):
+    import torch
+    nsm = torch.cuda.get_device_properties(0).multi_processor_count
+    last = nsm * dofs_per_sm // 2 ** dim          # most elements that take a lane per DOF
+    for n, variant in ((last, mdl.SWEEP_GROUP), (last + 1, mdl.SWEEP_THREAD)):
+        if n == 0:
+            continue
+        rows = max(k for k in range(1, 41) if n % k == 0)
+        base = (n // rows, rows, 1)
+        p = problem(dim, 1, precision, amr).replace(base=base, extent=(0.06 * base[0], 0.06 * base[1], 0.06),
+                                                    max_refine=depth, dt_barrier=0.0)
+        V = 0.5 + 0.5 * np.sin(np.arange(n * 2 ** dim) / 91.0)
+        a, b = mdl.Sim(p), mdl.Sim(p)
+        b.set_sweep_variant(variant)
+        for g in (a, b):
+            g.set_initial(V, 0.3 * V)
+            g.step_barriers(12)
+        assert np.array_equal(a.read_mesh()[1], b.read_mesh()[1])
+        assert np.array_equal(a.read_V(), b.read_V()) and np.array_equal(a.read_state(), b.read_state())
+        a.close()
+        b.close()
+
+
+@pytest.mark.parametrize("dim,precision", [(2, 32), (3, 32), (2, 64)])
+def test_adapting_run_does_not_depend_on_the_capacity(mdl, dim, precision):
+    """A context whose capacity grows during the run against one that had room from the start."""
+    base = (32, 32, 1) if dim == 2 else (16, 12, 8)
+    p = problem(dim, 1, precision, 1).replace(base=base, extent=tuple(b / 64.0 for b in base), max_refine=3, tau_refine=1e-12,
+                                              tau_coarsen=1e-13, dt_barrier=0.0, stimuli=[])
+    xy = [(i, j, k)[:dim] for k in range(base[2]) for j in range(base[1]) for i in range(base[0])]
+    roots = (np.zeros(len(xy), np.int8), np.array(xy, np.int32))
+    n1 = 2 ** dim                                   # every root's children, in Morton order
+    kids = (np.ones(len(xy) * n1, np.int8),
+            np.array([[2 * c[t] + ((b >> t) & 1) for t in range(dim)] for c in xy for b in range(n1)], np.int32))
+    small, large = mdl.Sim(p), mdl.Sim(p)
+    if dim == 2:                                    # level 2: 16384 leaves, capacity 32768
+        kids = (np.full(len(xy) * 16, 2, np.int8), np.array(
+            [(4 * i + (b & 1) + 2 * ((b >> 2) & 1), 4 * j + ((b >> 1) & 1) + 2 * ((b >> 3) & 1)) for i, j in xy for b in range(16)],
+            np.int32))
+    large.upload_mesh(*kids)
+    large.upload_mesh(*roots)
+    x = np.repeat(np.array(xy)[:, 0], 2 ** dim).astype(float)
+    V = 0.5 * (1.0 - np.tanh((x - 0.5 * base[0]) / 2.0))
+    for g in (small, large):
+        g.set_initial(V, np.zeros_like(V))
+        g.step_barriers(16)
+    assert small.sizes()[0] > 4096                  # the first capacity
+    for a, b in zip(small.read_mesh(), large.read_mesh()):
+        assert np.array_equal(a, b)
+    assert np.array_equal(small.read_V(), large.read_V()) and np.array_equal(small.read_state(), large.read_state())
+    small.close()
+    large.close()
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+def test_small_adapting_fp32_default_sweep_matches_the_thread_sweep(mdl, dim):
+    p = problem(dim, 1, 32, 1)
+    a, b = mdl.Sim(p), mdl.Sim(p)
+    b.set_sweep_variant(mdl.SWEEP_THREAD)
+    a.step_barriers(60)
+    b.step_barriers(60)
+    assert np.array_equal(a.read_mesh()[1], b.read_mesh()[1])
+    for x, y in ((a.read_V(), b.read_V()), (a.read_state(), b.read_state())):
+        assert np.abs(x - y).max() <= 2e-5 * max(np.abs(y).max(), 1e-30)
+    a.close()
+    b.close()
