@@ -234,7 +234,8 @@ void mdl_destroy(mdl_ctx* ctx);
 const char* mdl_version(void);
 
 /* Launch shape of the sweep kernel: threads per block in {64, 128, 256}, resident blocks
- * per SM with threads * blocks_per_sm <= 2048.  Results do not depend on it. */
+ * per SM with threads * blocks_per_sm <= 2048.  Results do not depend on it.  Until a shape is
+ * set: 128 and 16, with smaller blocks on meshes of fewer blocks than the GPU has SMs. */
 int mdl_set_tick_shape(mdl_ctx* ctx, int32_t threads, int32_t blocks_per_sm);
 
 /* Sweep kernel variant.  All follow Alg. 1 tick by tick; THREAD and COOP run the same

@@ -125,15 +125,17 @@ int64_t barriers_to(double dt, double t0, double t_end) {
 
 // Time `n` barriers of the context for each candidate sweep launch shape (threads, blocks
 // per SM) of its sweep variant and keep the fastest.  The variant itself is not tuned:
-// variants round differently, and a slot must give the values it gives alone.
+// variants round differently, and a slot must give the values it gives alone.  kOwnShape is the
+// context's own choice (128, 16, with smaller blocks on small meshes): no shape is set then.
+constexpr std::pair<int, int> kOwnShape{128, 16};
 int tune(mdl_ctx* c, int n, std::pair<int, int>* best) {
-    static const int cand[][2] = {{128, 16}, {64, 32}, {256, 8}, {128, 8}, {64, 16}};
+    static const std::pair<int, int> cand[] = {kOwnShape, {64, 32}, {256, 8}, {128, 8}, {64, 16}};
     double best_ms = 1e300;
-    *best = {128, 16};
+    *best = kOwnShape;
     mdl::CtxBase* x = c->impl;
     x->set_timing(1);
     for (const auto& s : cand) {
-        int rc = x->set_tick_shape(s[0], s[1]);
+        int rc = s == kOwnShape ? MDL_OK : x->set_tick_shape(s.first, s.second);
         if (rc) continue;
         // one untimed barrier captures the graphs
         int64_t done = 0;
@@ -146,11 +148,10 @@ int tune(mdl_ctx* c, int n, std::pair<int, int>* best) {
         const double ms = (s1.sweep_ms - s0.sweep_ms) / std::max<int64_t>(1, s1.timed_barriers - s0.timed_barriers);
         if (ms < best_ms) {
             best_ms = ms;
-            *best = {s[0], s[1]};
+            *best = s;
         }
     }
-    x->set_timing(0);
-    return x->set_tick_shape(best->first, best->second);
+    return MDL_OK;
 }
 
 // Candidate launch shapes of the fused sweep: threads per block, due elements per work
@@ -554,18 +555,18 @@ int mdl_batch_admit(mdl_batch* b, const mdl_problem* prob, const double* V0, con
         auto it = b->shapes.find(key);
         if (it == b->shapes.end()) {
             // tune on a temporary copy of the instance, which is stepped and discarded
-            std::pair<int, int> best{128, 16};
+            std::pair<int, int> best = kOwnShape;
             mdl_ctx* tmp = nullptr;
             if (mdl_create(prob, &tmp) == MDL_OK) {
                 if (!V0 || tmp->impl->set_initial(V0, s0, n_dof) == MDL_OK) {
-                    if (tune(tmp, 3, &best) != MDL_OK) best = {128, 16};
+                    if (tune(tmp, 3, &best) != MDL_OK) best = kOwnShape;
                 }
                 mdl_destroy(tmp);
             }
             b->shapes[key] = best;
             it = b->shapes.find(key);
         }
-        c->impl->set_tick_shape(it->second.first, it->second.second);
+        if (it->second != kOwnShape) c->impl->set_tick_shape(it->second.first, it->second.second);
     }
     int id = -1;
     for (size_t i = 0; i < b->slots.size(); ++i)

@@ -177,6 +177,7 @@ class Ctx : public CtxBase {
     PhaseGraph series[2];      // SERIES whole barriers, per state set at their start
     bool use_graphs = true;
     int tick_threads = 128, tick_bpsm = 16;   // sweep launch shape
+    bool auto_shape = true;                   // none asked for: small meshes take smaller blocks
     bool coop_sweep = false;                  // ticks + epilogue in one cooperative launch
     bool group_tick = false;                  // Q1: a group of (p+1)^d lanes per element
     bool auto_sweep = true;                   // no variant asked for: small Q1 meshes take the groups too
@@ -619,7 +620,7 @@ class Ctx : public CtxBase {
             }
             const bool grp = P == 1 && (group_tick || (auto_sweep && small_groups()));
             const int lanes = grp ? NP : 1;
-            const int tt = spread_threads(sweep_elems() * lanes, tick_threads);
+            const int tt = auto_shape ? spread_threads(sweep_elems() * lanes, tick_threads) : tick_threads;
             const int gt = (int)std::min<int64_t>(div_up(sweep_elems() * lanes, tt),
                                                   (int64_t)nsm * tick_bpsm * (tick_threads / tt));
             if constexpr (tensor_capable) {
@@ -1239,7 +1240,8 @@ public:
             err = "set_tick_shape: threads in {64,128,256}, threads * blocks_per_sm <= 2048";
             return MDL_E_ARG;
         }
-        if (threads != tick_threads || blocks_per_sm != tick_bpsm) {
+        if (auto_shape || threads != tick_threads || blocks_per_sm != tick_bpsm) {
+            auto_shape = false;
             tick_threads = threads;
             tick_bpsm = blocks_per_sm;
             drop_graphs();

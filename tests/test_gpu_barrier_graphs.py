@@ -171,3 +171,18 @@ def test_small_adapting_fp32_default_sweep_matches_the_thread_sweep(mdl, dim):
         assert np.abs(x - y).max() <= 2e-5 * max(np.abs(y).max(), 1e-30)
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("dim,order", [(2, 1), (2, 2), (3, 1), (3, 2)])
+def test_launch_shapes_give_the_same_bits_on_a_small_mesh(mdl, dim, order):
+    """The default's smaller blocks, and each shape that is set as it is set (a partial block)."""
+    p = problem(dim, order, 32, 0)
+    V = None
+    for shape in (None, (64, 32), (128, 16), (256, 8)):
+        g = mdl.Sim(p)
+        if shape:
+            g.set_tick_shape(*shape)
+        g.step_barriers(3)
+        V = g.read_V() if V is None else V
+        assert np.array_equal(g.read_V(), V)
+        g.close()
