@@ -389,7 +389,7 @@ def run_batch(args, rank, world):
     log-uniform in [1e3, 1e5], seed 4) stepped in fused rounds: a step is one batch round, every
     instance advancing one barrier; per element class the sweeps of all its instances run as
     one persistent launch per global tick, replayed from a captured graph, or as the
-    instances' own sweeps, whichever the batch's tuner measured faster during warm-up.  The K
+    instances' own sweeps, in whichever the batch's tuner measured the faster rounds during warm-up.  The K
     timed rounds are one batch step (issued back to back, waited for once).  One GPU: under a
     multi-rank launch it stops with an error instead of reporting one rank's rate."""
     if world > 1:
@@ -404,7 +404,7 @@ def run_batch(args, rank, world):
     slots = [b.admit(p, t_end) for p, t_end in inst]
     t_setup = time.perf_counter() - t_setup
     sims = {s: b.slot(s)[0] for s in slots}
-    # warm-up covers the tuner (7 candidates x 2 rounds per class, one round at a time)
+    # warm-up covers the tuner (14 rounds per class, one at a time)
     classes = ((32, 2, 1, "fp32_2d_q1"), (32, 3, 1, "fp32_3d_q1"), (32, 3, 2, "fp32_3d_q2"))
     warm = 0
     while warm < args.warmup or (not args.batch_streams and warm < 40 and
@@ -436,8 +436,8 @@ def run_batch(args, rank, world):
         if info:
             shapes[name] = {"choice": "own sweeps" if info["own"] else
                             "fused %d threads x %d elements per item" % (info["threads"], info["tile"]),
-                            "best_round_sweep_ms": round(info["best_ms"], 3),
-                            "worst_round_sweep_ms": round(info["worst_ms"], 3),
+                            "best_round_ms": round(info["best_ms"], 3),
+                            "worst_round_ms": round(info["worst_ms"], 3),
                             "own_sweeps_round_ms": round(info["own_ms"], 3)}
     out = {
         "metric": METRIC, "value": total / secs, "unit": UNIT, "n_gpus": world, "steps": args.steps,

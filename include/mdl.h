@@ -287,9 +287,10 @@ int mdl_set_sweep_blocks(mdl_ctx* ctx, int32_t max_blocks);
  *     tick (a slot with fewer LTS levels takes part in every 2^k-th), replayed from a CUDA
  *     graph captured for the batch's composition; then each slot's epilogue.  The rounds of
  *     one mdl_batch_step are issued back to back and waited for once.  With autotune the
- *     first rounds (one at a time) time, per class, every candidate launch shape of the
- *     fused kernel (threads per block, due elements per work item) and "own sweeps" (each
- *     slot's own sweep variant on its own stream) on the batch itself, and keep the fastest
+ *     first 14 rounds (one at a time) time, per class and on the batch itself, the sweeps of
+ *     six launch shapes of the fused kernel (threads per block, due elements per work item),
+ *     then whole rounds with the fastest of them against whole rounds of "own sweeps" (each
+ *     slot's barrier on its own stream with its own sweep variant), and keep the faster way
  *     (mdl_batch_fused_info); without autotune the fused kernel runs at 128 threads and 256
  *     due elements per work item.  A fused element takes the step of the thread-per-element
  *     sweep (MDL_SWEEP_THREAD): an instance gives the values it gives alone with that sweep,
@@ -328,9 +329,9 @@ int mdl_batch_set_fused(mdl_batch* b, int32_t on);
 /* Fused rounds so far and fused sweep kernel launches (rounds, launches: always written);
  * for the group of (precision 32|64, dim 2|3, order 1|2): own = 1 if the tuner chose each
  * slot's own sweep, else the tuned launch shape of the fused kernel (threads per block, due
- * elements per work item); the mean sweep time per round of the fastest and the slowest
- * candidate and of own sweeps, as the tuner measured them (MDL_E_STATE until tuned).  Any
- * output pointer may be NULL. */
+ * elements per work item); the time of a whole round of the batch, on the host's clock, in the
+ * faster and in the slower of the two ways and with own sweeps, as the tuner measured them
+ * (MDL_E_STATE until tuned).  Any output pointer may be NULL. */
 int mdl_batch_fused_info(const mdl_batch* b, int32_t precision, int32_t dim, int32_t order, int32_t* own,
                          int32_t* threads, int32_t* tile, double* best_ms, double* worst_ms, double* own_ms,
                          int64_t* rounds, int64_t* launches);

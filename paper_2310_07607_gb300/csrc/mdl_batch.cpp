@@ -9,10 +9,10 @@
 //     batch's composition (each class on its own stream, so the classes' sweeps overlap);
 //     then each slot's epilogue.  The rounds of one mdl_batch_step run
 //     back to back: the host waits for the device once, after the last.  Per class, the
-//     first rounds of the batch time every candidate on the batch itself -- launch shapes of
-//     the fused kernel (threads per block, due elements per work item) and "own sweeps"
-//     (each slot's own sweep variant on its own stream) -- and keep the fastest, counting what a
-//     fused round adds per slot.  A slot on its own runs its whole barrier as one graph.  A fused
+//     first rounds of the batch time launch shapes of the fused kernel (threads per block, due
+//     elements per work item) by their sweeps, then whole rounds with the fastest of them against
+//     whole rounds of "own sweeps" (each slot's own sweep variant on its own stream), and keep
+//     the faster way.  A slot on its own runs its whole barrier as one graph.  A fused
 //     element takes the step of the thread-per-element sweep, so an instance gives the values it
 //     gives alone with that sweep up to the FP32 rounding of the two kernels' compilations; with
 //     own sweeps it gives the bits it gives alone.
@@ -48,7 +48,6 @@ struct mdl_batch {
         int64_t barriers_done = 0;
         bool polled = false;
         int group = 0;          // fused group: (precision 64) * 4 + element class
-        bool own = false;       // this round's sweep: the slot's own (not the fused kernel)
     };
     int64_t budget = 0;
     int64_t used = 0;
@@ -84,13 +83,13 @@ struct mdl_batch {
         std::vector<Chunk> chunks;
         mdl::FusedShape shape{128, 256, 0};
         bool own = false;                         // tuned: each slot's own sweep
-        int tuned = 0;                            // candidate rounds timed so far (-1: done)
-        std::vector<double> cand_ms;              // measured ms per candidate
+        int tuned = 0;                            // tuning rounds so far (-1: done)
+        double shape_ms = 0;                      // sweep of the fastest shape so far
         cudaStream_t st = nullptr;                // the group's stream: its fused sweeps
         cudaEvent_t done = nullptr;               // the group's sweep of the round done
         cudaEvent_t t0 = nullptr, t1 = nullptr;   // tuner timing of the current round
         bool timed = false;
-        double best_ms = 0, worst_ms = 0, own_ms = 0;
+        double fused_ms = 0, own_ms = 0;          // whole rounds, the faster of two each
     };
     Group groups[8];                              // (precision 32 / 64) x element class
     int64_t fused_rounds = 0, fused_launches = 0;
@@ -154,19 +153,19 @@ int tune(mdl_ctx* c, int n, std::pair<int, int>* best) {
     return MDL_OK;
 }
 
-// Candidate launch shapes of the fused sweep: threads per block, due elements per work
-// item.  One more candidate follows them: each slot's own sweep on its own stream.
+// Tuning rounds of a group.  First one per candidate launch shape of the fused sweep (threads per
+// block, due elements per work item), timed by its sweep alone; then eight whole rounds, fused with
+// the fastest shape or every slot on its own.  The first two of either way are not counted (they
+// capture the graphs of an adapting slot's two state sets, 0.9 ms for 64 slots whose round takes
+// 0.22); the others take turns, and the faster round of each way decides.  Sweeps alone would not:
+// fused they are several times shorter, but a fused round adds a graph launch, an event and two stream
+// waits per slot on the host and the join of the group's slots.  Measured rounds, all fused / all
+// on their own, in us: 8, 24, 64 and 128 mixed instances 132 / 88, 622 / 460, 1608 / 1323,
+// 3050 / 2625; 8, 32 and 64 small adapting requests 208 / 121, 364 / 262, 470 / 384.
 const int kFusedShapes[][2] = {{128, 128}, {128, 512}, {256, 256}, {256, 1024}, {64, 256}, {128, 2048}};
-constexpr int kFusedCands = (int)(sizeof(kFusedShapes) / sizeof(kFusedShapes[0]));
-constexpr int kOwnCand = kFusedCands;
-constexpr int kCands = kFusedCands + 1;
-constexpr int kRoundsPerCand = 2;
-// What a fused round adds per slot beside its sweep: two graph launches instead of one and an event
-// with two stream waits on the host, and the join of the group's slots on the device.  Per round,
-// classes fused / all slots on their own: 8 small adapting requests 222 / 151 us, 24 mixed instances
-// 496 / 461 us, 8 of them 111 / 85 us, with sweeps of 0.13 ms fused against 0.20 to 0.28 ms own for
-// the 12 2D instances of the 24.
-constexpr double kFusedSlotMs = 0.03;
+constexpr int kShapes = (int)(sizeof(kFusedShapes) / sizeof(kFusedShapes[0]));
+constexpr char kWholeRounds[] = {'f', 'f', 'o', 'o', 'f', 'o', 'f', 'o'};
+constexpr int kWhole = (int)sizeof(kWholeRounds), kUncounted = 4;
 
 int sm_count() {
     int dev = 0, n = 1;
@@ -207,17 +206,23 @@ bool tuning(const mdl_batch* b) {
     return false;
 }
 
-// The candidate a group runs this round (-1: its tuned choice).
-int candidate(const mdl_batch* b, const mdl_batch::Group& g) {
-    return b->autotune && g.tuned >= 0 ? g.tuned / kRoundsPerCand : -1;
+// The shape whose sweep a group times this round (-1: none).
+int shape_trial(const mdl_batch* b, const mdl_batch::Group& g) {
+    return b->autotune && g.tuned >= 0 && g.tuned < kShapes ? g.tuned : -1;
+}
+
+// Whether a group's slots run on their own this round.
+bool own_round(const mdl_batch* b, const mdl_batch::Group& g) {
+    if (!b->autotune || g.tuned < 0) return g.own;
+    return g.tuned >= kShapes && kWholeRounds[g.tuned - kShapes] == 'o';
 }
 
 // Chunk c of the group's fused sweep of this round (records host[0 .. n), already holding
-// their shifts) from its captured graph, uploading the records and capturing first when
+// their shifts): its captured graph, uploading the records and capturing first when
 // they or the launch shape changed.  The group's pinned staging holds every chunk's records
 // at the chunk's own offset.
-int fused_group_sweep(mdl_batch* b, mdl_batch::Group& g, int c, const unsigned char* host, int n, int Bmax,
-                      int threads, int tile, int nsm) {
+int fused_group_graph(mdl_batch* b, mdl_batch::Group& g, int c, const unsigned char* host, int n, int Bmax,
+                      int threads, int tile, int nsm, cudaGraphExec_t* out) {
     const size_t bytes = mdl::fused_slot_bytes(g.precision);
     const size_t nb = (size_t)n * bytes;
     if ((int)g.chunks.size() <= c) g.chunks.resize(c + 1);
@@ -270,8 +275,7 @@ int fused_group_sweep(mdl_batch* b, mdl_batch::Group& g, int c, const unsigned c
         MDL_BCK(ei);
         E->key = key;
     }
-    MDL_BCK(cudaGraphLaunch(E->graph, g.st));
-    b->fused_launches += 1 << Bmax;
+    *out = E->graph;
     return MDL_OK;
 }
 
@@ -288,25 +292,24 @@ int fused_issue(mdl_batch* b, const std::vector<int>& run) {
         g.host.clear();
         g.timed = false;
     }
-    // the phases before the sweep, each slot on its own stream; a slot of a group tuned to own
-    // sweeps goes straight on to the end of its barrier
+    // the phases before the sweep, each slot on its own stream; a slot on its own goes straight on
+    // to the end of its barrier
     std::vector<int> Bs(b->slots.size(), 0);
     std::vector<int> begun;
     for (int i : run) {
         mdl_batch::Slot& s = b->slots[i];
         mdl_batch::Group& g = b->groups[s.group];
-        const int c = candidate(b, g);
         // a mapped slot always sweeps on its own and is no member of its group
         const bool alone = s.ctx->impl->is_mapped();
-        s.own = alone || (c >= 0 ? c == kOwnCand : g.own);
-        if (s.own && (c < 0 || alone)) {
+        if (alone || own_round(b, g)) {
             // nothing of the round is shared: the slot's whole barrier in one graph
             const int rc = s.ctx->impl->fused_whole();
             if (rc) {
                 s.state = MDL_SLOT_FAILED;
                 s.rc = rc;
+            } else if (!alone) {
+                g.members.push_back(i);
             }
-            if (!alone) g.members.push_back(i);
             continue;
         }
         const size_t bytes = mdl::fused_slot_bytes(g.precision);
@@ -324,19 +327,36 @@ int fused_issue(mdl_batch* b, const std::vector<int>& run) {
         begun.push_back(i);
     }
     // per (precision, class) group, on the group's own stream (the groups' sweeps overlap):
-    // one fused sweep from its captured graph, or (timed while tuning) the slots' own sweeps.
-    // While tuning, the groups' sweeps run one after another so that each is timed alone.
+    // one fused sweep from its captured graph.  While shapes are timed, the groups' sweeps run one
+    // after another so that each is timed alone.
     const int nsm = sm_count();
-    const bool serial = tuning(b);
+    bool serial = false;
+    for (const auto& g : b->groups) serial = serial || (!g.members.empty() && shape_trial(b, g) >= 0);
     cudaEvent_t prev = nullptr;
+    std::vector<cudaGraphExec_t> sweeps;
     for (auto& g : b->groups) {
         const int n = (int)g.members.size();
-        if (n == 0) continue;
-        const int c = candidate(b, g);
-        if (c < 0 && g.own) continue;
+        if (n == 0 || own_round(b, g)) continue;
+        const int c = shape_trial(b, g);
         if (!g.st) {
             MDL_BCK(cudaStreamCreateWithFlags(&g.st, cudaStreamNonBlocking));
             MDL_BCK(cudaEventCreateWithFlags(&g.done, cudaEventDisableTiming));
+        }
+        const size_t bytes = mdl::fused_slot_bytes(g.precision);
+        const int threads = c >= 0 ? kFusedShapes[c][0] : g.shape.threads;
+        const int tile = c >= 0 ? kFusedShapes[c][1] : g.shape.tile;
+        sweeps.clear();
+        for (int c0 = 0, ci = 0; c0 < n; c0 += mdl::FUSED_MAX_SLOTS, ++ci) {
+            const int nc = std::min(n - c0, mdl::FUSED_MAX_SLOTS);
+            int Bmax = 0;
+            for (int k = c0; k < c0 + nc; ++k) Bmax = std::max(Bmax, Bs[g.members[k]]);
+            for (int k = c0; k < c0 + nc; ++k)
+                mdl::fused_set_shift(g.host.data() + k * bytes, g.precision, Bmax - Bs[g.members[k]]);
+            cudaGraphExec_t sweep = nullptr;
+            const int rc = fused_group_graph(b, g, ci, g.host.data() + c0 * bytes, nc, Bmax, threads, tile, nsm, &sweep);
+            if (rc) return rc;
+            sweeps.push_back(sweep);
+            b->fused_launches += 1 << Bmax;
         }
         for (int i : g.members) MDL_BCK(cudaStreamWaitEvent(g.st, b->sev[i], 0));
         if (serial && prev) MDL_BCK(cudaStreamWaitEvent(g.st, prev, 0));
@@ -348,33 +368,7 @@ int fused_issue(mdl_batch* b, const std::vector<int>& run) {
             MDL_BCK(cudaEventRecord(g.t0, g.st));
             g.timed = true;
         }
-        if (c == kOwnCand) {
-            for (int i : g.members) {
-                mdl_batch::Slot& s = b->slots[i];
-                cudaStream_t ss = (cudaStream_t)s.ctx->impl->stream_handle();
-                MDL_BCK(cudaStreamWaitEvent(ss, g.t0, 0));
-                const int rc = s.ctx->impl->fused_own_sweep();
-                if (rc) {
-                    s.state = MDL_SLOT_FAILED;
-                    s.rc = rc;
-                }
-                MDL_BCK(cudaEventRecord(b->sev[i], ss));
-                MDL_BCK(cudaStreamWaitEvent(g.st, b->sev[i], 0));
-            }
-        } else {
-            const size_t bytes = mdl::fused_slot_bytes(g.precision);
-            const int threads = c >= 0 ? kFusedShapes[c][0] : g.shape.threads;
-            const int tile = c >= 0 ? kFusedShapes[c][1] : g.shape.tile;
-            for (int c0 = 0, ci = 0; c0 < n; c0 += mdl::FUSED_MAX_SLOTS, ++ci) {
-                const int nc = std::min(n - c0, mdl::FUSED_MAX_SLOTS);
-                int Bmax = 0;
-                for (int k = c0; k < c0 + nc; ++k) Bmax = std::max(Bmax, Bs[g.members[k]]);
-                for (int k = c0; k < c0 + nc; ++k)
-                    mdl::fused_set_shift(g.host.data() + k * bytes, g.precision, Bmax - Bs[g.members[k]]);
-                const int rc = fused_group_sweep(b, g, ci, g.host.data() + c0 * bytes, nc, Bmax, threads, tile, nsm);
-                if (rc) return rc;
-            }
-        }
+        for (cudaGraphExec_t sweep : sweeps) MDL_BCK(cudaGraphLaunch(sweep, g.st));
         if (c >= 0) MDL_BCK(cudaEventRecord(g.t1, g.st));
         MDL_BCK(cudaEventRecord(g.done, g.st));
         prev = g.done;
@@ -382,8 +376,7 @@ int fused_issue(mdl_batch* b, const std::vector<int>& run) {
     // each slot's epilogue after its sweep
     for (int i : begun) {
         mdl_batch::Slot& s = b->slots[i];
-        if (s.state == MDL_SLOT_FAILED) continue;
-        if (!s.own) MDL_BCK(cudaStreamWaitEvent((cudaStream_t)s.ctx->impl->stream_handle(), b->groups[s.group].done, 0));
+        MDL_BCK(cudaStreamWaitEvent((cudaStream_t)s.ctx->impl->stream_handle(), b->groups[s.group].done, 0));
         const int rc = s.ctx->impl->fused_finish();
         if (rc) {
             s.state = MDL_SLOT_FAILED;
@@ -394,8 +387,7 @@ int fused_issue(mdl_batch* b, const std::vector<int>& run) {
     return MDL_OK;
 }
 
-// Wait for the rounds issued since the last completion: complete every slot that took part
-// and, while tuning, add the round's timings to the candidates (after the last, keep the best).
+// Wait for the rounds issued since the last completion: complete every slot that took part.
 int fused_complete(mdl_batch* b, const std::vector<char>& took_part, int64_t* total) {
     for (size_t i = 0; i < b->slots.size(); ++i) {
         mdl_batch::Slot& s = b->slots[i];
@@ -406,27 +398,28 @@ int fused_complete(mdl_batch* b, const std::vector<char>& took_part, int64_t* to
     }
     for (auto& g : b->groups)
         if (g.st) MDL_BCK(cudaStreamSynchronize(g.st));
+    return MDL_OK;
+}
+
+// One tuning round of every group that took part in it is complete; round_ms: from its first launch
+// to its completion on the host.
+int tune_round(mdl_batch* b, double round_ms) {
     for (auto& g : b->groups) {
-        if (!g.timed) continue;
-        g.timed = false;
-        float ms = 0;
-        MDL_BCK(cudaEventElapsedTime(&ms, g.t0, g.t1));
-        const int c = g.tuned / kRoundsPerCand;
-        if ((int)g.cand_ms.size() < kCands) g.cand_ms.assign(kCands, 0.0);
-        g.cand_ms[c] += ms;
-        if (++g.tuned == kCands * kRoundsPerCand) {
-            // the fastest fused shape, unless the slots' own sweeps cost less with what a fused round
-            // adds per slot
-            int best = 0;
-            for (int k = 1; k < kFusedCands; ++k)
-                if (g.cand_ms[k] < g.cand_ms[best]) best = k;
-            const double extra = kFusedSlotMs * (double)g.members.size() * kRoundsPerCand;
-            g.own = g.cand_ms[kOwnCand] <= g.cand_ms[best] + extra;
-            const double least = *std::min_element(g.cand_ms.begin(), g.cand_ms.end());
-            if (!g.own) g.shape = mdl::FusedShape{kFusedShapes[best][0], kFusedShapes[best][1], 0};
-            g.best_ms = least / kRoundsPerCand;
-            g.worst_ms = *std::max_element(g.cand_ms.begin(), g.cand_ms.end()) / kRoundsPerCand;
-            g.own_ms = g.cand_ms[kOwnCand] / kRoundsPerCand;
+        if (!b->autotune || g.tuned < 0 || g.members.empty()) continue;
+        if (g.timed) {
+            g.timed = false;
+            float ms = 0;
+            MDL_BCK(cudaEventElapsedTime(&ms, g.t0, g.t1));
+            if (g.tuned == 0 || ms < g.shape_ms) {
+                g.shape_ms = ms;
+                g.shape = mdl::FusedShape{kFusedShapes[g.tuned][0], kFusedShapes[g.tuned][1], 0};
+            }
+        } else if (g.tuned - kShapes >= kUncounted) {
+            double& m = own_round(b, g) ? g.own_ms : g.fused_ms;
+            m = m > 0 ? std::min(m, round_ms) : round_ms;
+        }
+        if (++g.tuned == kShapes + kWhole) {
+            g.own = g.own_ms <= g.fused_ms;
             g.tuned = -1;
         }
     }
@@ -459,6 +452,7 @@ int fused_step(mdl_batch* b, int64_t rounds, int64_t* total) {
         }
         if (run.empty()) break;
         const bool sync_each = tuning(b);
+        const auto t0 = std::chrono::steady_clock::now();
         int rc = fused_issue(b, run);
         for (int i : run) {
             took[i] = 1;
@@ -471,6 +465,8 @@ int fused_step(mdl_batch* b, int64_t rounds, int64_t* total) {
         }
         if (sync_each || tuning(b)) {
             if ((rc = fused_complete(b, took, total))) return rc;
+            const std::chrono::duration<double, std::milli> ms = std::chrono::steady_clock::now() - t0;
+            if ((rc = tune_round(b, ms.count()))) return rc;
             std::fill(took.begin(), took.end(), 0);
             pending = false;
             // horizons and failures as of this completion
@@ -736,8 +732,8 @@ int mdl_batch_fused_info(const mdl_batch* b, int32_t precision, int32_t dim, int
     if (own) *own = g.own ? 1 : 0;
     if (threads) *threads = g.shape.threads;
     if (tile) *tile = g.shape.tile;
-    if (best_ms) *best_ms = g.best_ms;
-    if (worst_ms) *worst_ms = g.worst_ms;
+    if (best_ms) *best_ms = std::min(g.fused_ms, g.own_ms);
+    if (worst_ms) *worst_ms = std::max(g.fused_ms, g.own_ms);
     if (own_ms) *own_ms = g.own_ms;
     return MDL_OK;
 }

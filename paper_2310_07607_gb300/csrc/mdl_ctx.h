@@ -43,13 +43,11 @@ public:
     // Fused batch rounds (mdl_fused.h): launch the phases before the sweep (indicator,
     // adaptation, levels, ordering) of one barrier on the context's stream and write the
     // slot's sweep record (a FusedSlot of the context's precision, shift left 0) and its LTS
-    // level count B; after the batch's fused sweep (or after fused_own_sweep(), the
-    // context's own sweep variant on its own stream), launch the epilogue.  Several rounds
+    // level count B; after the batch's fused sweep, launch the epilogue.  Several rounds
     // may be issued before end_barriers(), which then completes them as after
     // begin_barriers(rounds).  A context with replayed inputs (set_levels, set_indicators)
     // takes one round per end_barriers(); replaying() says so.
     virtual int fused_begin(void* slot_record, int* B) = 0;
-    virtual int fused_own_sweep() = 0;
     virtual int fused_finish() = 0;
     // A whole round of a slot that sweeps on its own: every phase of one barrier on its stream (in
     // place of fused_begin .. fused_finish).

@@ -155,7 +155,6 @@ class Ctx : public CtxBase {
     DBuf<Phys<R>> dph;
     DBuf<OpT<R, DIM, P>> dop;
     int fused_cur = 0;        // state set the fused sweep of the barrier in flight updates
-    bool fused_own = false;   // this round's sweep is the context's own (fused_own_sweep)
     DevMeta* hmeta = nullptr;
     bool ovr_levels = false, ovr_eta_s = false, ovr_eta_t = false;
     bool timing = false;
@@ -1292,7 +1291,6 @@ public:
             return MDL_E_STATE;
         }
         if (!inflight) inflight_start = nbar;
-        fused_own = false;
         const int o = cs;
         int rc;
         if ((rc = run_phases(first_phase(), 1, o, direct))) return rc;
@@ -1305,14 +1303,6 @@ public:
         fs->cls = DIM == 2 ? (P == 1 ? FC_2_1 : FC_2_2) : (P == 1 ? FC_3_1 : FC_3_2);
         fs->shift = 0;
         if (Bout) *Bout = B;
-        return MDL_OK;
-    }
-
-    int fused_own_sweep() override {
-        const bool direct = ovr_levels || ovr_eta_s || ovr_eta_t;
-        int rc = run_phases(2, 2, cs, direct);
-        if (rc) return rc;
-        fused_own = true;
         return MDL_OK;
     }
 
@@ -1330,11 +1320,8 @@ public:
 
     int fused_finish() override {
         const bool direct = ovr_levels || ovr_eta_s || ovr_eta_t;
-        // the cooperative sweep runs the epilogue itself
-        if (!(fused_own && coop_sweep)) {
-            int rc = run_phases(3, 3, cs, direct);
-            if (rc) return rc;
-        }
+        int rc = run_phases(3, 3, cs, direct);
+        if (rc) return rc;
         cs = fused_cur;
         inflight += 1;
         return MDL_OK;

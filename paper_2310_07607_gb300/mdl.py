@@ -422,8 +422,8 @@ class Batch:
 
     def fused_info(self, precision: int = 32, dim: int = 2, order: int = 1):
         """The tuner's choice for the (precision, dim, order) group -- a dict with "own" (each
-        slot's own sweep) or the fused kernel's "threads" and "tile", and the measured
-        "best_ms", "worst_ms" and "own_ms" per round -- or None before the tuner finished;
+        slot's own sweep) or the fused kernel's "threads" and "tile", and the measured whole
+        rounds "best_ms", "worst_ms" (the two ways) and "own_ms" -- or None before the tuner finished;
         and the batch's fused (rounds, launches)."""
         own, t, k = C.c_int32(), C.c_int32(), C.c_int32()
         bm, wm, om = C.c_double(), C.c_double(), C.c_double()

@@ -248,3 +248,21 @@ def test_fused_group_larger_than_one_launch(mdl):
     for s in slots:
         b.release(s)
     b.close()
+
+
+def test_the_tuner_keeps_the_way_of_the_faster_rounds(mdl):
+    """The choice between the fused sweep and the slots' own ones is the one whose measured rounds were
+    the faster, for a handful and for many small instances of one class."""
+    for n in (6, 48):
+        b = mdl.Batch(autotune=True, fused=True)
+        slots = [b.admit(instance(2, 1, i % 5), 1e6) for i in range(n)]
+        b.step(barriers_per_slot=13)
+        assert b.fused_info(32, 2, 1)[0] is None
+        b.step(barriers_per_slot=1)
+        info, (rounds, _) = b.fused_info(32, 2, 1)
+        assert rounds == 14
+        assert info["own_ms"] in (info["best_ms"], info["worst_ms"]) and info["best_ms"] <= info["worst_ms"]
+        assert info["own"] == (info["own_ms"] == info["best_ms"])
+        for s in slots:
+            b.release(s)
+        b.close()
