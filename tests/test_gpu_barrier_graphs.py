@@ -142,8 +142,8 @@ def test_adapting_run_does_not_depend_on_the_capacity(mdl, dim, precision):
     small, large = mdl.Sim(p), mdl.Sim(p)
     if dim == 2:                                    # level 2: 16384 leaves, capacity 32768
         kids = (np.full(len(xy) * 16, 2, np.int8), np.array(
-            [(4 * i + (b & 1) + 2 * ((b >> 2) & 1), 4 * j + ((b >> 1) & 1) + 2 * ((b >> 3) & 1)) for i, j in xy for b in range(16)],
-            np.int32))
+            [(4 * i + (b & 1) + 2 * ((b >> 2) & 1), 4 * j + ((b >> 1) & 1) + 2 * ((b >> 3) & 1)) for i, j in xy
+             for b in range(16)], np.int32))
     large.upload_mesh(*kids)
     large.upload_mesh(*roots)
     x = np.repeat(np.array(xy)[:, 0], 2 ** dim).astype(float)
@@ -154,6 +154,32 @@ def test_adapting_run_does_not_depend_on_the_capacity(mdl, dim, precision):
     assert small.sizes()[0] > 4096                  # the first capacity
     for a, b in zip(small.read_mesh(), large.read_mesh()):
         assert np.array_equal(a, b)
+    assert np.array_equal(small.read_V(), large.read_V()) and np.array_equal(small.read_state(), large.read_state())
+    small.close()
+    large.close()
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+def test_curved_run_does_not_depend_on_the_capacity(mdl, precision):
+    """The factors of curved elements lie in groups of 32 elements: they keep their places when the
+    arrays grow.  The context with room has been refined everywhere and coarsened to its roots before."""
+    base = (24, 10, 2)
+    p = W.lv_3d_q1_amr(base).replace(precision=precision, tau_refine=1e-12, tau_coarsen=1e-13, stimuli=[])
+    xyz = [(i, j, k) for k in range(base[2]) for j in range(base[1]) for i in range(base[0])]
+    small, large = mdl.Sim(p), mdl.Sim(p)
+    peak = 0
+    for eta in (1.0, 1.0, 0.0, 0.0):
+        large.set_indicators(eta_s=np.full(large.sizes()[0], eta))
+        large.step_barriers(1)
+        peak = max(peak, large.sizes()[0])
+    assert peak == 64 * len(xyz) and large.sizes()[0] == len(xyz)
+    V = np.repeat(0.5 * (1.0 - np.tanh((np.array(xyz)[:, 0] - 12.0) / 2.0)), 8)
+    for g in (small, large):
+        g.set_initial(V, np.zeros_like(V))
+        g.step_barriers(5)
+    assert small.sizes()[0] > 4096
+    for x, y in zip(small.read_mesh(), large.read_mesh()):
+        assert np.array_equal(x, y)
     assert np.array_equal(small.read_V(), large.read_V()) and np.array_equal(small.read_state(), large.read_state())
     small.close()
     large.close()
