@@ -851,9 +851,9 @@ def main():
     ap.add_argument("--tick-shape", default="", help="sweep launch shape 'threads,blocks_per_sm'")
     ap.add_argument("--base", default="", help="base grid 'nx,ny[,nz]' at the workload's element size")
     ap.add_argument("--sweep", default="default", choices=["default"] + sorted(SWEEPS),
-                    help="sweep kernel variant (default: the library's choice, thread; "
-                         "thread otherwise; thread per element; group: Q1 lanes per element; coop: one "
-                         "cooperative launch per barrier; tensor: tcgen05 residual, Q2 3D FP32)")
+                    help="sweep kernel variant (default: the library's choice; thread: a thread per element; "
+                         "group: Q1, a lane per DOF; coop: one cooperative launch per barrier; "
+                         "tensor: tcgen05 residual, Q2 3D FP32)")
     args = ap.parse_args()
     if args.warmup < 3:
         args.warmup = 3

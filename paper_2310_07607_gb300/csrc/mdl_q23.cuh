@@ -1,7 +1,7 @@
 // mdl_q23.cuh -- the sweep tick of Q2 3D FP32 contexts (MDL_SWEEP_THREAD, their default).
 //
 // A thread per due element, with the operator of mdl_boxop.cuh (about 1,000 multiply-adds) and
-// ap_step (about 1,300 operations for the 27 DOFs).  A step reads the element's row of 27 values
+// ap_step (about 1,450 operations for the 27 DOFs).  A step reads the element's row of 27 values
 // and six neighbour rows, and the element's state and barrier-start rows.  Loaded by the thread
 // that uses them these are 16-byte accesses to 32 rows per instruction, whose 32 cache lines the
 // L1 looks up one by one.  So a warp copies its rows together: 7 consecutive lanes take one row

@@ -228,7 +228,8 @@ class Sim:
         self._check(self.lib.mdl_set_tick_shape(self.h, threads, blocks_per_sm))
 
     def set_sweep_variant(self, variant: int):
-        """SWEEP_THREAD (the default), SWEEP_GROUP (Q1), SWEEP_COOP or SWEEP_TENSOR (Q2 3D FP32)."""
+        """SWEEP_THREAD (the default but for small Q1 contexts), SWEEP_GROUP (Q1; theirs), SWEEP_COOP or
+        SWEEP_TENSOR (Q2 3D FP32)."""
         self._check(self.lib.mdl_set_sweep_variant(self.h, variant))
 
     def set_sweep_blocks(self, max_blocks: int):
